@@ -32,6 +32,7 @@
 namespace kifmm {
 
 int tc_tile_pairs(int Qp);
+int tc_row_groups(int Mr);
 int tc_split_table(const float* table, __half* hi, __half* lo, size_t n, int* texp, cudaStream_t s);
 int tc_box_split(const float* v, int Q, int Qp, int b0, int b1, __half* hi, __half* lo, int* e, cudaStream_t s);
 int tc_make_map(CUtensorMap* map, const __half* table, int nops, int Mr, int Kp);
@@ -1414,6 +1415,34 @@ void sort_by_op(std::vector<Triple>& tr) {
     tr.swap(out);
 }
 
+// Pairs per tile of one tensor-core launch over the pairs tr, at most cap.  The launch's
+// CTAs (one per SM) take its items in turn, and an item costs a fixed part (kTileFixed, in
+// columns: the operator's rows and the pipeline's latency per stage of K -- an item of 16
+// columns measured 1.4 k clk a stage, one of 128 2.5 k) plus its columns.  The cap with the
+// least (items per CTA) x (item cost) is taken: a launch of few pairs (coarse levels, small
+// trees) spreads over more SMs in narrow tiles, a large one keeps whole tiles.
+constexpr int kTileFixed = 160;
+int tile_cap(const std::vector<Triple>& tr, int cap, int mgroups, int nsm) {
+    if (nsm <= 0) return cap;
+    std::vector<int> cnt;
+    for (const Triple& x : tr) {
+        if ((size_t)x.op >= cnt.size()) cnt.resize((size_t)x.op + 1, 0);
+        ++cnt[(size_t)x.op];
+    }
+    int best = cap;
+    int64_t best_cost = INT64_MAX;
+    for (int c = cap; c >= 16; c -= 16) {
+        int64_t items = 0;
+        for (int n : cnt) items += (n + c - 1) / c;
+        const int64_t cost = (items * mgroups + nsm - 1) / nsm * (kTileFixed + c);
+        if (cost < best_cost) {
+            best_cost = cost;
+            best = c;
+        }
+    }
+    return best;
+}
+
 void make_tiles(std::vector<Triple>& tr, std::vector<int4>& tiles, std::vector<int>& pin,
                 std::vector<int>& pout, int cap) {
     sort_by_op(tr);
@@ -1515,7 +1544,7 @@ void m2l_schedule(std::vector<Triple>& tr, const std::vector<int>& level, int ca
     for (size_t i = 0; i < tr.size(); ++i)
         if (!chained[i]) rest.push_back(tr[i]);
     if (chains.empty()) {
-        make_tiles(rest, tiles, pin, pout, cap);
+        make_tiles(rest, tiles, pin, pout, tile_cap(rest, cap, 1, G));
         return;
     }
     std::vector<int4> single;
@@ -1982,6 +2011,16 @@ int setup(Plan& P, const double* src_nrm, const double* trg_nrm, cudaStream_t s)
     // CUDA-core blocks of kPairTile
     const int cap_up = P.fp64 ? kPairTile : tc_tile_pairs(P.ops->Ku);
     const int cap_dn = P.fp64 ? kPairTile : tc_tile_pairs(P.ops->Kd);
+    int nsm = 0;                    // mixed: the SMs the tiles of a launch are spread over
+    if (!P.fp64) {
+        int dev = 0;
+        KF_CHECK_CUDA(cudaGetDevice(&dev));
+        KF_CHECK_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    }
+    // pairs per tile of a launch whose operators have Mr rows (mixed; FP64: the cap)
+    auto cap_for = [&](const std::vector<Triple>& tr, int cap, int Mr) {
+        return tile_cap(tr, cap, P.fp64 ? 1 : tc_row_groups(Mr), nsm);
+    };
     if (!P.fp64) {
         const int kz = std::max(P.ops->Ku, P.ops->Kd);
         KF_TRY(P.bexp.alloc(T.nbox));
@@ -2345,7 +2384,7 @@ int setup(Plan& P, const double* src_nrm, const double* trg_nrm, cudaStream_t s)
                         if (c >= 0 && has_src(T, c)) tr.push_back({o, c, b});
                     }
                 }
-                make_tiles(tr, tiles, pin, pout, cap_up);
+                make_tiles(tr, tiles, pin, pout, cap_for(tr, cap_up, P.ops->Ku));
             }
         }
         P.u2u.level_tile[T.nlev] = (int)tiles.size();
@@ -2368,14 +2407,11 @@ int setup(Plan& P, const double* src_nrm, const double* trg_nrm, cudaStream_t s)
         // covers all of an operator's rows (Kd <= 256) and the kernel runs one CTA per SM
         P.m2l_chain_pairs = 0;
         if (!P.fp64 && P.ops->Kd <= 256) {
-            int dev = 0, nsm = 0;
-            KF_CHECK_CUDA(cudaGetDevice(&dev));
-            KF_CHECK_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
             std::vector<int> kcount;
             m2l_schedule(tr, T.h_lvl, cap_dn, nsm, tiles, pin, pout, kcount, &P.m2l_chain_pairs);
             if (!kcount.empty()) KF_TRY(P.m2l.kcount.upload(kcount, s));
         } else {
-            make_tiles(tr, tiles, pin, pout, cap_dn);
+            make_tiles(tr, tiles, pin, pout, cap_for(tr, cap_dn, P.ops->Kd));
         }
         KF_TRY(upload_tiles(P.m2l, tiles, pin, pout, s));
     }
@@ -2390,7 +2426,7 @@ int setup(Plan& P, const double* src_nrm, const double* trg_nrm, cudaStream_t s)
                 std::vector<Triple> tr;
                 for (int b = T.level_off[l]; b < T.level_off[l + 1]; ++b)
                     if (has_trg(T, b)) tr.push_back({octant_of(T, b), T.h_parent[b], b});
-                make_tiles(tr, tiles, pin, pout, cap_dn);
+                make_tiles(tr, tiles, pin, pout, cap_for(tr, cap_dn, P.ops->Kd));
             }
         }
         P.l2l.level_tile[T.nlev] = (int)tiles.size();
@@ -2405,7 +2441,7 @@ int setup(Plan& P, const double* src_nrm, const double* trg_nrm, cudaStream_t s)
             std::vector<int> pin, pout;
             std::vector<Triple> tr;
             for (int b : up ? s2u_box : p2l_box) tr.push_back({0, b, b});
-            make_tiles(tr, tiles, pin, pout, up ? cap_up : cap_dn);
+            make_tiles(tr, tiles, pin, pout, cap_for(tr, up ? cap_up : cap_dn, up ? P.ops->Ku : P.ops->Kd));
             KF_TRY(upload_tiles(up ? P.proj_up : P.proj_x, tiles, pin, pout, s));
         }
         KF_TRY(P.zu.alloc((size_t)T.nbox * P.ops->Ku));

@@ -92,6 +92,7 @@ int get_encoder(EncodeTiled* fn) {
 // Operator rows per work item and pairs per tile for operators of Mr (padded) rows.
 int tc_rows(int Mr) { return Mr <= 128 ? 128 : 256; }
 int tc_tile_pairs(int Mr) { return Mr <= 128 ? 256 : 128; }
+int tc_row_groups(int Mr) { return (Mr + tc_rows(Mr) - 1) / tc_rows(Mr); }
 
 // Scale an FP32 operator table by 2^texp (largest entry into [2^14, 2^15)) and split it
 // into FP16 hi and lo tables.  Synchronizes the stream (texp is needed on the host).
@@ -153,6 +154,15 @@ static int launch_shape(int which, const CUtensorMap& hi, const CUtensorMap& lo,
                              : tc::k_proj_tc<SLABS, N>;
     // set on every launch: the attribute belongs to the current device's context
     KF_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kSmemBytes));
+    // the kernel's register split draws on kLaunchRegs a thread: with fewer its fold warps
+    // would wait for registers that never come
+    cudaFuncAttributes fa;
+    KF_CHECK_CUDA(cudaFuncGetAttributes(&fa, kern));
+    if (fa.numRegs < tc::kLaunchRegs) {
+        set_error("translation kernel built with %d registers a thread, its register split needs %d", fa.numRegs,
+                  tc::kLaunchRegs);
+        return KIFMM_ERR_UNSUPPORTED;
+    }
     const int mgroups = (Mr + S::kRows - 1) / S::kRows;
     const int nitems = ntiles * mgroups;
     // persistent: one CTA per SM (one fits by shared memory), each walking its share of
