@@ -519,89 +519,6 @@ int launch_surf(const Plan& P, const Tree& T, bool dl, int nbox, const int* boxe
     return KIFMM_OK;
 }
 
-// ---------------------------------------------------------------- grouped pair GEMM (U2U, M2L, L2L)
-// Every tile shares one operator: out[pout[j]] += Op . in[pin[j]] for its pairs.
-// CUDA-core SGEMM/DGEMM blocking: 64 rows x 64 pairs per pass, 4x4 per thread.
-template <typename Real>
-__device__ __forceinline__ void pair_gemm_body(const Real* __restrict__ ops, int Q, int Qp,
-                                               const int4* __restrict__ tiles, const int* __restrict__ pin,
-                                               const int* __restrict__ pout, const Real* __restrict__ in,
-                                               Real* __restrict__ out) {
-    constexpr int BM = 64, BN = kPairTile, BK = 16;
-    __shared__ Real As[BK][BM + 4];
-    __shared__ Real Bs[BK][BN + 4];
-    __shared__ int s_in[BN], s_out[BN];
-    int4 t = tiles[blockIdx.x];
-    const Real* Op = ops + (size_t)t.x * Qp * Qp;
-    int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-    for (int jb = 0; jb < t.z; jb += BN) {  // tiles may hold several blocks of BN pairs
-    const int cnt = t.z - jb;
-    __syncthreads();
-    for (int j = threadIdx.x; j < BN; j += blockDim.x) {
-        s_in[j] = j < cnt ? pin[t.y + jb + j] : -1;
-        s_out[j] = j < cnt ? pout[t.y + jb + j] : -1;
-    }
-    __syncthreads();
-    for (int row0 = 0; row0 < Q; row0 += BM) {
-        Real acc[4][4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) acc[i][j] = 0;
-        for (int k0 = 0; k0 < Qp; k0 += BK) {
-            for (int e = threadIdx.x; e < BM * BK; e += blockDim.x) {
-                int r = e / BK, kk = e % BK;
-                int row = row0 + r;
-                As[kk][r] = row < Qp ? Op[(size_t)row * Qp + k0 + kk] : (Real)0;
-            }
-            for (int e = threadIdx.x; e < BN * BK; e += blockDim.x) {
-                int j = e / BK, kk = e % BK;
-                int bi = s_in[j];
-                Bs[kk][j] = bi >= 0 ? in[(size_t)bi * Qp + k0 + kk] : (Real)0;
-            }
-            __syncthreads();
-#pragma unroll
-            for (int kk = 0; kk < BK; ++kk) {
-                Real a[4], bv[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) a[i] = As[kk][ty * 4 + i];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) bv[j] = Bs[kk][tx * 4 + j];
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) acc[i][j] += a[i] * bv[j];
-            }
-            __syncthreads();
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            int row = row0 + ty * 4 + i;
-            if (row >= Q) continue;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                int ob = s_out[tx * 4 + j];
-                if (ob >= 0) atomicAdd(&out[(size_t)ob * Qp + row], acc[i][j]);
-            }
-        }
-    }
-    }
-}
-
-// One kernel name per translation so profiles tell them apart.
-#define KF_PAIR_KERNEL(NAME)                                                                              \
-    template <typename Real>                                                                              \
-    __global__ void __launch_bounds__(256)                                                               \
-        NAME(const Real* __restrict__ ops, int Q, int Qp, const int4* __restrict__ tiles,                \
-             const int* __restrict__ pin, const int* __restrict__ pout, const Real* __restrict__ in,     \
-             Real* __restrict__ out) {                                                                    \
-        pair_gemm_body<Real>(ops, Q, Qp, tiles, pin, pout, in, out);                                      \
-    }
-KF_PAIR_KERNEL(k_u2u_gemm)
-KF_PAIR_KERNEL(k_m2l_gemm)
-KF_PAIR_KERNEL(k_l2l_gemm)
-#undef KF_PAIR_KERNEL
-
 // ---------------------------------------------------------------- mean removal (ADL)
 // The adjoint double layer needs only the gradient of the far field.  A constant
 // potential has none, so each box's down-check potential is shifted to zero mean
@@ -1812,11 +1729,61 @@ int build_projected(Plan& P, const HostPinv& h, OpTables* t, const std::vector<d
     return KIFMM_OK;
 }
 
-// Per-target evaluation rows G(x_t, 2.95 s) P: P = Pd (Q wide, stored Qp) or, factored,
-// Wd (rd wide, stored Kd).
-template <typename Real>
-int build_d2t(Plan& P, const HostPinv& h, bool factored, int Kd, const std::vector<int>& tleaf_of, int axis,
-              Real* out, cudaStream_t s) {
+// Per-target evaluation rows of the mixed form, G(x_t, 2.95 s) W_d (rd wide, stored Kd):
+// an FP64 product (W_d carries factors 1 / sigma, and its terms cancel to O(1)), rounded
+// once to FP32.  The kernel values of a chunk of targets are written as exact slices and
+// multiplied on the tensor cores (sliced.cuh): 98,000 targets at p = 10 took 21.7 ms as FP64
+// FMAs at the FP64 pipe's rate.  A chunk is 64 targets per SM: whole waves of the kernel, and
+// slices that stay in L2.
+int build_d2t_sliced(Plan& P, const HostPinv& h, const std::vector<int>& tleaf_of, float* out, cudaStream_t s) {
+    const Tree& T = P.tree->t;
+    const int64_t nt = T.nt;
+    if (nt == 0) return KIFMM_OK;
+    const int Kd = P.ops->Kd;
+    int dev = 0, nsm = 0;
+    KF_CHECK_CUDA(cudaGetDevice(&dev));
+    KF_CHECK_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    const int chunk = (int)std::min<int64_t>(nt, (int64_t)nsm * kSlicePairs);
+    std::vector<double> hb(3 * (size_t)h.Q);
+    for (size_t i = 0; i < hb.size(); ++i) hb[i] = kDnEquiv * h.surf[i];
+    std::vector<int> iota(chunk);
+    std::iota(iota.begin(), iota.end(), 0);
+    // the tiles of a full chunk, then those of the last, partial one
+    std::vector<int4> tiles;
+    auto add_tiles = [&](int n) {
+        for (int i = 0; i < n; i += kSlicePairs) tiles.push_back(make_int4(0, i, std::min(kSlicePairs, n - i), 0));
+    };
+    add_tiles(chunk);
+    const int nfull = (int)tiles.size(), rest = (int)(nt % chunk);
+    add_tiles(rest);
+    DBuf<int> dleaf, dio, dexp;
+    DBuf<double> bpts, dos;
+    DBuf<int4> dtiles;
+    DBuf<__half> sl;
+    KF_TRY(dleaf.upload(tleaf_of, s));
+    KF_TRY(bpts.upload(hb, s));
+    KF_TRY(dio.upload(iota, s));
+    KF_TRY(dtiles.upload(tiles, s));
+    KF_TRY(dexp.alloc(chunk));
+    KF_TRY(dos.alloc(chunk));
+    KF_TRY(sl.alloc((size_t)chunk * slice_cols(h.Q) * kSlices));
+    const double* txyz = T.same ? T.sxyz.p : T.txyz.p;
+    const double* tn = P.kernel == KIFMM_KERNEL_ADL ? P.tnrm_d.p : nullptr;
+    for (int c = 0; c < P.nc; ++c)
+        for (int64_t t0 = 0; t0 < nt; t0 += chunk) {
+            const int n = (int)std::min<int64_t>(chunk, nt - t0);
+            KF_TRY(slice_eval_rows(dleaf.p, t0, n, nt, txyz, tn, c, T.lvl.p, T.ctr.p, T.root_h, bpts.p, h.Q,
+                                   gradient_kernel(P.kernel), sl.p, dexp.p, dos.p, s));
+            KF_TRY(launch_sliced_store<float>(P.ops->wd, P.ops->rd, n == chunk ? dtiles.p : dtiles.p + nfull,
+                                              div_up(n, kSlicePairs), dio.p, dio.p, sl.p, dexp.p, dos.p,
+                                              out + ((size_t)c * nt + t0) * Kd, Kd, P.err.p, s));
+        }
+    KF_CHECK_CUDA(cudaStreamSynchronize(s));   // the scratch is freed on return
+    return KIFMM_OK;
+}
+
+// The same of the FP64 form, G(x_t, 2.95 s) Pd (Q wide, stored Qp).
+int build_d2t(Plan& P, const HostPinv& h, const std::vector<int>& tleaf_of, int axis, double* out, cudaStream_t s) {
     const Tree& T = P.tree->t;
     int64_t nt = T.nt;
     DBuf<int> dleaf;
@@ -1830,8 +1797,7 @@ int build_d2t(Plan& P, const HostPinv& h, bool factored, int Kd, const std::vect
     std::vector<double> hb(3 * (size_t)h.Q);
     for (size_t i = 0; i < hb.size(); ++i) hb[i] = kDnEquiv * h.surf[i];
     KF_TRY(bpts.upload(hb, s));
-    KF_TRY(dPd.upload(factored ? h.Wd : h.Pd, s));
-    const int C = factored ? h.rd : P.Q, Kc = factored ? Kd : P.Qp;
+    KF_TRY(dPd.upload(h.Pd, s));
     const double* txyz = T.same ? T.sxyz.p : T.txyz.p;
     const bool adl = gradient_kernel(P.kernel);
     const double* tn = P.kernel == KIFMM_KERNEL_ADL ? P.tnrm_d.p : nullptr;
@@ -1849,7 +1815,7 @@ int build_d2t(Plan& P, const HostPinv& h, bool factored, int Kd, const std::vect
         rs.bset = nullptr;
         rs.orow = orow.p + r0;
         rs.bpts = bpts.p;
-        KF_TRY(build_rows<Real>(rs, P.Q, C, Kc, dPd.p, adl ? 1 : 0, out, s));
+        KF_TRY(build_rows<double>(rs, P.Q, P.Q, P.Qp, dPd.p, adl ? 1 : 0, out, s));
     }
     KF_CHECK_CUDA(cudaStreamSynchronize(s));
     return KIFMM_OK;
@@ -1891,18 +1857,20 @@ int get_tables(Plan& P, const HostPinv& h, cudaStream_t s) {
     t->centered = centered;
     const size_t QQ = (size_t)P.Qp * P.Qp;
     if (P.fp64) {
-        KF_TRY(t->m2m_d.alloc(8 * QQ));
-        KF_TRY(t->m2l_d.alloc(kNumOffsets * QQ));
-        KF_TRY(t->l2l_d.alloc(8 * QQ));
-        KF_CHECK_CUDA(cudaMemsetAsync(t->m2m_d.p, 0, t->m2m_d.bytes(), s));
-        KF_CHECK_CUDA(cudaMemsetAsync(t->m2l_d.p, 0, t->m2l_d.bytes(), s));
-        KF_CHECK_CUDA(cudaMemsetAsync(t->l2l_d.p, 0, t->l2l_d.bytes(), s));
+        DBuf<double> f64[3];
+        const int nops[3] = {8, kNumOffsets, 8};
+        for (int f = 0; f < 3; ++f) {
+            KF_TRY(f64[f].alloc(nops[f] * QQ));
+            KF_CHECK_CUDA(cudaMemsetAsync(f64[f].p, 0, f64[f].bytes(), s));
+        }
         t->ru = P.cheb ? P.Q : h.ru;
         t->rd = P.cheb ? P.Q : h.rd;
         if (P.cheb)
-            KF_TRY(build_cheb_ops(P, t->m2m_d.p, t->m2l_d.p, t->l2l_d.p, s));
+            KF_TRY(build_cheb_ops(P, f64[0].p, f64[1].p, f64[2].p, s));
         else
-            KF_TRY(build_ops(P, h, t->m2m_d.p, t->m2l_d.p, t->l2l_d.p, s));
+            KF_TRY(build_ops(P, h, f64[0].p, f64[1].p, f64[2].p, s));
+        for (int f = 0; f < 3; ++f) KF_TRY(slice_table(f64[f].p, nops[f], P.Qp, P.Q, P.Qp, t->fp64_ops[f], s));
+        KF_CHECK_CUDA(cudaStreamSynchronize(s));   // the FP64 tables are freed here
     } else {
         // translations between projections (see build_projected), two-term FP16
         t->ru = h.ru;
@@ -1948,6 +1916,14 @@ int get_tables(Plan& P, const HostPinv& h, cudaStream_t s) {
             KF_TRY(tc_make_map(&t->tmaps[f][0], t->tab_h[f].p, nops[f], rows[f], cols[f]));
             KF_TRY(tc_make_map(&t->tmaps[f][1], t->tab_l[f].p, nops[f], rows[f], cols[f]));
         }
+        // W_d^T, the factor of the evaluation rows (build_d2t_sliced)
+        std::vector<double> wt((size_t)t->Kd * h.Q, 0.0);
+        for (int i = 0; i < h.Q; ++i)
+            for (int j = 0; j < h.rd; ++j) wt[(size_t)j * h.Q + i] = h.Wd[(size_t)i * h.rd + j];
+        DBuf<double> dwt;
+        KF_TRY(dwt.upload(wt, s));
+        KF_TRY(slice_table(dwt.p, 1, t->Kd, h.Q, h.Q, t->wd, s));
+        KF_CHECK_CUDA(cudaStreamSynchronize(s));
     }
     KF_CHECK_CUDA(cudaStreamSynchronize(s));
     P.ops = t;
@@ -2008,7 +1984,7 @@ int setup(Plan& P, const double* src_nrm, const double* trg_nrm, cudaStream_t s)
     KF_TRY(get_tables(P, h, s));
     KF_TRY(stamp(0));
     // mixed: tiles sized for the tensor-core GEMM of each family's row count; FP64:
-    // CUDA-core blocks of kPairTile
+    // tiles of the sliced GEMM
     const int cap_up = P.fp64 ? kPairTile : tc_tile_pairs(P.ops->Ku);
     const int cap_dn = P.fp64 ? kPairTile : tc_tile_pairs(P.ops->Kd);
     int nsm = 0;                    // mixed: the SMs the tiles of a launch are spread over
@@ -2470,8 +2446,10 @@ int setup(Plan& P, const double* src_nrm, const double* trg_nrm, cudaStream_t s)
             KF_CHECK_CUDA(cudaStreamSynchronize(s));
         } else {
             for (int c = 0; c < P.nc; ++c)
-                KF_TRY(build_d2t<double>(P, h, false, 0, tleaf_of, c, P.d2t_d.p + (size_t)c * T.nt * P.Qp, s));
+                KF_TRY(build_d2t(P, h, tleaf_of, c, P.d2t_d.p + (size_t)c * T.nt * P.Qp, s));
         }
+        KF_TRY(P.bexp.alloc(T.nbox));
+        KF_TRY(P.vsl.alloc((size_t)T.nbox * slice_cols(P.Q) * kSlices));
         KF_TRY(P.u_d.alloc(nbq));
         KF_TRY(P.d_d.alloc(nbq));
         KF_TRY(P.res_d.alloc((size_t)P.nc * T.nt));
@@ -2479,8 +2457,7 @@ int setup(Plan& P, const double* src_nrm, const double* trg_nrm, cudaStream_t s)
     } else {
         // rows G W_d, reading the projected down-check potentials
         KF_TRY(P.d2t_f.alloc((size_t)P.nc * T.nt * P.ops->Kd));
-        for (int c = 0; c < P.nc; ++c)
-            KF_TRY(build_d2t<float>(P, h, true, P.ops->Kd, tleaf_of, c, P.d2t_f.p + (size_t)c * T.nt * P.ops->Kd, s));
+        KF_TRY(build_d2t_sliced(P, h, tleaf_of, P.d2t_f.p, s));
         // (no FP32 check potentials: S2U and X write the projections' split inputs)
         KF_TRY(P.res_f.alloc((size_t)P.nc * T.nt));
         // DL: the dipoles q n_j as FP32 and their FP32 remainders (6 rows); else 3 rows
@@ -2493,7 +2470,7 @@ int setup(Plan& P, const double* src_nrm, const double* trg_nrm, cudaStream_t s)
     for (size_t b : {(size_t)P.ops->bytes(), P.d2t_d.bytes(), P.d2t_f.bytes(), P.u_d.bytes(), P.d_d.bytes(),
                      P.res_d.bytes(), P.q_d.bytes(), P.u_f.bytes(), P.d_f.bytes(), P.res_f.bytes(),
                      P.q_f.bytes(), P.snrm.bytes(), P.tnrm_d.bytes(), P.tnrm_f.bytes(),
-                     P.bexp.bytes(), P.vin_h.bytes(), P.vin_l.bytes(), P.sexp.bytes(), P.sin_h.bytes(),
+                     P.bexp.bytes(), P.vsl.bytes(), P.vin_h.bytes(), P.vin_l.bytes(), P.sexp.bytes(), P.sin_h.bytes(),
                      P.sin_l.bytes(), P.sxf.bytes(), P.txf.bytes(), P.bcf.bytes(), P.zu.bytes(),
                      P.zd.bytes()})
         P.device_bytes += (int64_t)b;
@@ -2567,17 +2544,19 @@ int project(const Plan& P, int fam, const PairTiles& pt, float* z, cudaStream_t 
     return KIFMM_OK;
 }
 
-// FP64: CUDA-core blocked GEMM.
+// FP64: exact FP16 slices on the tensor cores (sliced.cuh); the inputs of the launch (boxes
+// [b0, b1)) are sliced first.
 template <>
 int run_pairs<double>(const Plan& P, int which, const PairTiles& pt, int t0, int t1, const double* ops,
                       const double* in, double* out, int b0, int b1, cudaStream_t s, int& launches) {
-    (void)b0;
-    (void)b1;
-    using Real = double;
+    (void)ops;
+    if (b1 > b0) {
+        KF_TRY(slice_vectors(in, P.Q, P.Qp, b0, b1, P.vsl.p, P.bexp.p, s));
+        ++launches;
+    }
     if (t1 <= t0) return KIFMM_OK;
-    auto kern = which == kU2U ? k_u2u_gemm<Real> : which == kM2L ? k_m2l_gemm<Real> : k_l2l_gemm<Real>;
-    kern<<<t1 - t0, 256, 0, s>>>(ops, P.Q, P.Qp, pt.tiles.p + t0, pt.pin.p, pt.pout.p, in, out);
-    KF_CHECK_LAUNCH();
+    KF_TRY(launch_sliced_add(P.ops->fp64_ops[which], P.Q, pt.tiles.p + t0, t1 - t0, pt.pin.p, pt.pout.p, P.vsl.p, P.bexp.p,
+                             out, P.Qp, P.err.p, s));
     ++launches;
     return KIFMM_OK;
 }
@@ -2826,7 +2805,7 @@ int matvec(Plan& P, const Bufs<Real>& B, const double* q, double* out, cudaStrea
 
 int plan_matvec(Plan& P, const double* q, double* out, cudaStream_t s) {
     if (P.fp64) {
-        Bufs<double> B{P.ops->m2m_d.p, P.ops->m2l_d.p, P.ops->l2l_d.p, P.d2t_d.p, P.surf_d.p, P.tnrm_d.p,
+        Bufs<double> B{nullptr, nullptr, nullptr, P.d2t_d.p, P.surf_d.p, P.tnrm_d.p,
                        P.u_d.p,   P.d_d.p,   P.res_d.p, P.q_d.p};
         return matvec<double>(P, B, q, out, s);
     }

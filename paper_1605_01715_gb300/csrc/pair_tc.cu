@@ -123,23 +123,28 @@ int tc_box_split(const float* v, int Q, int Qp, int b0, int b1, __half* hi, __ha
     return KIFMM_OK;
 }
 
-// 2-D tiled map over rows (op * Mr + row) x columns (Kp) of an FP16 table, box kKS
-// columns x tc_rows(Mr) rows, 64-byte swizzle, zero fill outside.
-int tc_make_map(CUtensorMap* map, const __half* table, int nops, int Mr, int Kp) {
+// 2-D tiled map of a row-major FP16 matrix, box kKS columns x box_rows rows, 64-byte
+// swizzle, zero fill outside.
+int tc_make_map_rows(CUtensorMap* map, const __half* p, int64_t nrows, int Kp, int box_rows) {
     EncodeTiled enc;
     KF_TRY(get_encoder(&enc));
-    cuuint64_t dims[2] = {(cuuint64_t)Kp, (cuuint64_t)nops * (cuuint64_t)Mr};
+    cuuint64_t dims[2] = {(cuuint64_t)Kp, (cuuint64_t)nrows};
     cuuint64_t strides[1] = {(cuuint64_t)Kp * sizeof(__half)};
-    cuuint32_t box[2] = {(cuuint32_t)tc::kKS, (cuuint32_t)tc_rows(Mr)};
+    cuuint32_t box[2] = {(cuuint32_t)tc::kKS, (cuuint32_t)box_rows};
     cuuint32_t estr[2] = {1, 1};
-    CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<__half*>(table), dims, strides, box, estr,
+    CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<__half*>(p), dims, strides, box, estr,
                      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) {
-        set_error("cuTensorMapEncodeTiled failed (%d) for a %d x %d table", (int)r, nops * Mr, Kp);
+        set_error("cuTensorMapEncodeTiled failed (%d) for a %lld x %d table", (int)r, (long long)nrows, Kp);
         return KIFMM_ERR_CUDA;
     }
     return KIFMM_OK;
+}
+
+// Operator tables: rows (op * Mr + row), boxes of tc_rows(Mr) rows.
+int tc_make_map(CUtensorMap* map, const __half* table, int nops, int Mr, int Kp) {
+    return tc_make_map_rows(map, table, (int64_t)nops * Mr, Kp, tc_rows(Mr));
 }
 
 template <int SLABS, int N>

@@ -8,6 +8,7 @@
 #include <memory>
 
 #include "common.cuh"
+#include "sliced.cuh"
 
 namespace kifmm {
 
@@ -20,7 +21,7 @@ struct PairTiles {
     int64_t npairs = 0;
 };
 
-constexpr int kPairTile = 64;
+constexpr int kPairTile = kSlicePairs;     // FP64: pairs per translation tile
 // events per profiled matvec: 0..8 bound the 8 phases on the matvec's stream (8 = end),
 // 9 and 10 bound the near field (on the near-field stream when it overlaps the far field)
 constexpr int kPhaseEvents = 11;
@@ -49,12 +50,14 @@ struct OpTables {
     int ru = 0, rd = 0, Ku = 0, Kd = 0;
     int ks = 0;                     // mixed: S2U points (skeleton of the up-check surface)
     DBuf<float> surf_up;            // mixed: those points on the unit surface, ks x 3
-    DBuf<double> m2m_d, m2l_d, l2l_d;
+    SlicedTable fp64_ops[3];        // FP64: M2M', M2L', L2L' in exact slices (see sliced.cuh)
+    SlicedTable wd;                 // mixed: W_d^T (rd of Kd rows), the evaluation rows' factor
     DBuf<__half> tab_h[kFamilies], tab_l[kFamilies];
     int texp[kFamilies] = {0, 0, 0, 0, 0};
     CUtensorMap tmaps[kFamilies][2];
     int64_t bytes() const {
-        int64_t b = m2m_d.bytes() + m2l_d.bytes() + l2l_d.bytes() + surf_up.bytes();
+        int64_t b = wd.bytes() + surf_up.bytes();
+        for (const SlicedTable& t : fp64_ops) b += t.bytes();
         for (int f = 0; f < kFamilies; ++f) b += tab_h[f].bytes() + tab_l[f].bytes();
         return b;
     }
@@ -80,6 +83,7 @@ struct Plan {
     DBuf<float> d2t_f;
     DBuf<int> bexp, sexp;
     DBuf<__half> vin_h, vin_l, sin_h, sin_l;
+    DBuf<__half> vsl;               // FP64: the check potentials a translation reads, sliced (exponents in bexp)
     DBuf<double> surf_d;            // Q x 3 unit surface
     DBuf<float> surf_f;
 
