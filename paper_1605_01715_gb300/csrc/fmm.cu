@@ -587,25 +587,27 @@ k_d2t(const int* __restrict__ leaves, const int64_t* __restrict__ rng, const Rea
 // KIND 0: q/r   1: (q n_j).(x - y)/r^3   2: q n_i.(x - y)/r^3   3: q (x - y)/r^3 (three
 // components, written to out[tperm[t] + c nt] with the far field res[t + c nt])
 template <typename Real, int KIND>
-__global__ void k_p2p(const int* __restrict__ leaves, const int* __restrict__ off, const int* __restrict__ idx,
-                      const int64_t* __restrict__ rng, const double* __restrict__ ctr,
-                      const double* __restrict__ sxyz, int64_t ns, const double* __restrict__ txyz,
-                      int64_t nt, const Real* __restrict__ qs, const Real* __restrict__ tnrm,
-                      const Real* __restrict__ res, const int64_t* __restrict__ tperm,
+__global__ void k_p2p(const int* __restrict__ order, const int* __restrict__ leaves, const int* __restrict__ off,
+                      const longlong2* __restrict__ ranges, const int64_t* __restrict__ rng,
+                      const double* __restrict__ ctr, const double* __restrict__ sxyz, int64_t ns,
+                      const double* __restrict__ txyz, int64_t nt, const Real* __restrict__ qs,
+                      const Real* __restrict__ tnrm, const Real* __restrict__ res, const int64_t* __restrict__ tperm,
                       double* __restrict__ out) {
-    extern __shared__ unsigned char smem_raw[];
-    Real* sx = reinterpret_cast<Real*>(smem_raw);
-    Real* sy = sx + blockDim.x;
-    Real* sz = sy + blockDim.x;
-    Real* s0 = sz + blockDim.x;
-    Real* s1 = s0 + blockDim.x;
-    Real* s2 = s1 + blockDim.x;
-    int b = leaves[blockIdx.x];
-    double cx = ctr[3 * b], cy = ctr[3 * b + 1], cz = ctr[3 * b + 2];
-    int64_t tb = rng[4 * b + 2], te = rng[4 * b + 3];
+    using R4 = typename Vec4<Real>::T;
+    using R2 = typename Vec4<Real>::T2;
+    extern __shared__ __align__(32) unsigned char smem_raw[];
+    R4* sp = reinterpret_cast<R4*>(smem_raw);                    // two chunks of (x, y, z, q)
+    R2* sd = reinterpret_cast<R2*>(sp + 2 * blockDim.x);        // KIND 1: the dipoles' other components
+    const int li = order[blockIdx.x], b = leaves[li];
+    const double cx = ctr[3 * b], cy = ctr[3 * b + 1], cz = ctr[3 * b + 2];
+    const int64_t tb = rng[4 * b + 2], te = rng[4 * b + 3];
+    const int nthr = (int)(te - tb < (int64_t)blockDim.x ? (te - tb + 31) / 32 * 32 : (int64_t)blockDim.x);
+    const int ti = threadIdx.x;
+    if (ti >= nthr) return;                                      // whole warps; barriers below count nthr
+    const int e0 = off[li], e1 = off[li + 1];
     const Real d2 = (Real)(kDelta * kDelta);
-    for (int64_t t0 = tb; t0 < te; t0 += blockDim.x) {
-        int64_t t = t0 + threadIdx.x;
+    for (int64_t t0 = tb; t0 < te; t0 += nthr) {
+        int64_t t = t0 + ti;
         bool valid = t < te;
         int64_t tt = valid ? t : tb;
         Real xt = (Real)(txyz[tt] - cx), yt = (Real)(txyz[nt + tt] - cy), zt = (Real)(txyz[2 * nt + tt] - cz);
@@ -616,48 +618,42 @@ __global__ void k_p2p(const int* __restrict__ leaves, const int* __restrict__ of
             nz = tnrm[2 * nt + tt];
         }
         Real acc = 0, acc2 = 0, acc3 = 0;
-        for (int e = off[blockIdx.x]; e < off[blockIdx.x + 1]; ++e) {
-            int a = idx[e];
-            int64_t sb = rng[4 * a], se = rng[4 * a + 1];
-            for (int64_t j0 = sb; j0 < se; j0 += blockDim.x) {
-                int64_t j = j0 + threadIdx.x;
-                if (j < se) {
-                    sx[threadIdx.x] = (Real)(sxyz[j] - cx);
-                    sy[threadIdx.x] = (Real)(sxyz[ns + j] - cy);
-                    sz[threadIdx.x] = (Real)(sxyz[2 * ns + j] - cz);
-                    s0[threadIdx.x] = qs[j];
-                    if (KIND == 1) {
-                        s1[threadIdx.x] = qs[ns + j];
-                        s2[threadIdx.x] = qs[2 * ns + j];
-                    }
+        // the position in the ranges; the range after the current one is loaded ahead
+        int e = e0;
+        longlong2 cur = e0 < e1 ? ranges[e0] : make_longlong2(0, 0);
+        longlong2 nxt = e0 + 1 < e1 ? ranges[e0 + 1] : make_longlong2(0, 0);
+        double gx = 0, gy = 0, gz = 0;
+        Real g0 = 0, g1 = 0, g2 = 0;
+        auto fetch = [&]() -> int {                              // the next chunk's sources to registers
+            int got = 0;
+            int64_t j = -1;
+            while (e < e1 && got < nthr) {
+                const int n = (int)(cur.y - cur.x < nthr - got ? cur.y - cur.x : nthr - got);
+                if (ti >= got && ti < got + n) j = cur.x + (ti - got);
+                got += n;
+                cur.x += n;
+                if (cur.x >= cur.y) {
+                    cur = nxt;
+                    ++e;
+                    if (e + 1 < e1) nxt = ranges[e + 1];
                 }
-                __syncthreads();
-                int cnt = (int)((se - j0) < (int64_t)blockDim.x ? (se - j0) : (int64_t)blockDim.x);
-                for (int jj = 0; jj < cnt; ++jj) {
-                    Real dx = xt - sx[jj], dy = yt - sy[jj], dz = zt - sz[jj];
-                    Real r2 = dx * dx + dy * dy + dz * dz;
-                    Real inv = RT<Real>::rsq(r2);
-                    Real v;
-                    if (KIND == 3) {
-                        const Real w = (r2 >= d2) ? s0[jj] * (inv * inv * inv) : (Real)0;
-                        acc += w * dx;
-                        acc2 += w * dy;
-                        acc3 += w * dz;
-                        continue;
-                    }
-                    if (KIND == 0) v = s0[jj] * inv;
-                    else if (KIND == 1) v = (s0[jj] * dx + s1[jj] * dy + s2[jj] * dz) * (inv * inv * inv);
-                    else v = s0[jj] * (nx * dx + ny * dy + nz * dz) * (inv * inv * inv);
-                    acc += (r2 >= d2) ? v : (Real)0;
+            }
+            if (j >= 0) {
+                gx = sxyz[j];
+                gy = sxyz[ns + j];
+                gz = sxyz[2 * ns + j];
+                g0 = qs[j];
+                if (KIND == 1) {
+                    g1 = qs[ns + j];
+                    g2 = qs[2 * ns + j];
                 }
-                __syncthreads();
             }
         }
         if (valid) {
-            out[tperm[t]] = (double)(acc + res[t]);
+            out[tperm[t]] = (double)(res ? acc + res[t] : acc);
             if (KIND == 3) {
-                out[tperm[t] + nt] = (double)(acc2 + res[t + nt]);
-                out[tperm[t] + 2 * nt] = (double)(acc3 + res[t + 2 * nt]);
+                out[tperm[t] + nt] = (double)(res ? acc2 + res[t + nt] : acc2);
+                out[tperm[t] + 2 * nt] = (double)(res ? acc3 + res[t + 2 * nt] : acc3);
             }
         }
     }
@@ -678,7 +674,61 @@ __global__ void k_p2p(const int* __restrict__ leaves, const int* __restrict__ of
 // shared-memory broadcast, every value already duplicated as a float2 pair.
 //
 // Accuracy (Sec. III.A.1 asks for the discrete sum; these are the steps that keep the
+            return got;
+        };
+        auto term = [&](const R4& y, const R2* yd, Real& dx, Real& dy, Real& dz, Real& w, Real& v) {
+            dx = xt - y.x, dy = yt - y.y, dz = zt - y.z;
+            const Real r2 = dx * dx + dy * dy + dz * dz;
+            const Real inv = RT<Real>::rsq(r2);
+            w = v = 0;
+            if (KIND == 3) {
+                w = (r2 >= d2) ? y.w * (inv * inv * inv) : (Real)0;
+                return;
+            }
+            if (KIND == 0) v = y.w * inv;
+            else if (KIND == 1) v = (y.w * dx + yd->x * dy + yd->y * dz) * (inv * inv * inv);
+            else v = y.w * (nx * dx + ny * dy + nz * dz) * (inv * inv * inv);
+            v = (r2 >= d2) ? v : (Real)0;
+        };
+        auto add = [&](Real dx, Real dy, Real dz, Real w, Real v) {
+            if (KIND == 3) {
+                acc += w * dx;
+                acc2 += w * dy;
+                acc3 += w * dz;
+            } else {
+                acc += v;
+            }
+        };
+        constexpr int kU = std::is_same<Real, float>::value ? 8 : 4;
+        int cnt = fetch(), buf = 0;
+        while (cnt > 0) {
+            R4* p = sp + buf * blockDim.x;
+            R2* q = sd + buf * blockDim.x;
+            p[ti] = R4{(Real)(gx - cx), (Real)(gy - cy), (Real)(gz - cz), g0};
+            if (KIND == 1) q[ti] = R2{g1, g2};
+            asm volatile("bar.sync 1, %0;" ::"r"(nthr) : "memory");
+            const int ncnt = fetch();
+            // kU sources in flight per thread (the heaviest leaf's warps run alone on their
+            // schedulers, so the latency of one source's chain is what they wait for); their
+            // terms are added in order
+            int jj = 0;
+            for (; jj + kU <= cnt; jj += kU) {
+                Real dx[kU], dy[kU], dz[kU], w[kU], v[kU];
+#pragma unroll
+                for (int u = 0; u < kU; ++u) term(p[jj + u], q + jj + u, dx[u], dy[u], dz[u], w[u], v[u]);
+#pragma unroll
+                for (int u = 0; u < kU; ++u) add(dx[u], dy[u], dz[u], w[u], v[u]);
+            }
+            for (; jj < cnt; ++jj) {
+                Real dx, dy, dz, w, v;
+                term(p[jj], q + jj, dx, dy, dz, w, v);
+                add(dx, dy, dz, w, v);
+            }
+            buf ^= 1;
+            cnt = ncnt;
 // FP32 evaluation at the single layer's accuracy for all three kernels):
+        // the last chunk is read before the next pass stages its first
+        asm volatile("bar.sync 1, %0;" ::"r"(nthr) : "memory");
 //  - Offsets are taken from the leaf centre.  Each range has an exponent E with every
 //    coordinate offset of the leaf's targets and the range's sources below 2^E (from
 //    the boxes' extents).  For the double layers an offset is split as hi + lo, hi on the
@@ -715,9 +765,8 @@ constexpr int kCloseBits = 5;
 __host__ __device__ inline int range_exp(long long fl) { return (int)((fl >> 48) & 255) - 128; }
 constexpr int kP2PUnitSrc = 2048;
 // Larger target leaves of the single layer and the field go to the block kernel (a
-// thread per target, sources staged once per leaf): at leaf 128 on the 64-sphere pack it
-// takes 2.56 ms against 4.04 ms for two 64-target passes of the warp kernel.  The double
-// layers always take the warp kernel, in passes, for its exact products.
+// thread per target, sources staged once per leaf).  The double layers always take the
+// warp kernel, in passes, for its exact products.
 constexpr int kP2PWarpMaxLeaf = 64;
 // unit flags (int4 .w): bit 0 the leaf's first unit, bit 1 the leaf spans several units;
 // bits 8..9 the dipoles' axis of a KIND 4 unit; bits 16..30 one plus the unit's one pass
@@ -2139,7 +2188,22 @@ int setup(Plan& P, const double* src_nrm, const double* trg_nrm, cudaStream_t s)
     KF_TRY(P.p2l_idx.upload(p2l_idx, s));
     KF_TRY(P.tleaf.upload(tleaf, s));
     KF_TRY(P.p2p_off.upload(p2p_off, s));
-    KF_TRY(P.p2p_idx.upload(p2p_idx, s));
+    // the block kernel's source ranges and its leaves, heaviest first
+    if (!warp_near(P)) {
+        std::vector<longlong2> lr(p2p_idx.size());
+        std::vector<int64_t> work(tleaf.size(), 0);
+        for (size_t li = 0; li < tleaf.size(); ++li)
+            for (int k = p2p_off[li]; k < p2p_off[li + 1]; ++k) {
+                const int a = p2p_idx[k];
+                lr[k] = make_longlong2(T.h_rng[4 * a], T.h_rng[4 * a + 1]);
+                work[li] += lr[k].y - lr[k].x;
+            }
+        std::vector<int> ord(tleaf.size());
+        std::iota(ord.begin(), ord.end(), 0);
+        std::stable_sort(ord.begin(), ord.end(), [&](int x, int y) { return work[x] > work[y]; });
+        KF_TRY(P.p2p_lranges.upload(lr, s));
+        KF_TRY(P.p2p_order.upload(ord, s));
+    }
     if (!P.fp64 && !box_ax.empty()) {
         std::vector<int> hbax(T.nbox, 3);
         // 4 + k: every source of the box in one plane normal to its dipoles' axis k
@@ -2626,10 +2690,10 @@ int matvec(Plan& P, const Bufs<Real>& B, const double* q, double* out, cudaStrea
         }
         if (!done) {
         int threads = std::min(256, std::max(32, (P.max_trg_leaf + 31) / 32 * 32));
-        size_t smem = 6 * threads * sizeof(Real);
+        size_t smem = 2 * (size_t)threads * 6 * sizeof(Real);
 #define KF_P2P(KIND)                                                                                     \
-    k_p2p<Real, KIND><<<P.n_tleaf, threads, smem, ns>>>(P.tleaf.p, P.p2p_off.p, P.p2p_idx.p, T.rng.p,     \
-                                                        T.ctr.p, T.sxyz.p, T.ns, txyz, T.nt, B.q, B.tnrm, \
+    k_p2p<Real, KIND><<<P.n_tleaf, threads, smem, ns>>>(P.p2p_order.p, P.tleaf.p, P.p2p_off.p, P.p2p_lranges.p, T.rng.p, \
+                                                        T.ctr.p, T.sxyz.p, T.ns, txyz, T.nt, B.q, B.tnrm,          \
                                                         res, tperm, out)
         if (P.kernel == KIFMM_KERNEL_SL) KF_P2P(0);
         else if (P.kernel == KIFMM_KERNEL_DL) KF_P2P(1);
@@ -2643,8 +2707,7 @@ int matvec(Plan& P, const Bufs<Real>& B, const double* q, double* out, cudaStrea
     };
     // mixed, warp near field: it runs on its own stream beside the far field (forked
     // after the gather) and the far field is added once both are done
-    const bool near_overlap = std::is_same<Real, float>::value && P.n_tleaf && P.near_stream && warp_near(P) &&
-                              !P.serial;
+    const bool near_overlap = std::is_same<Real, float>::value && P.n_tleaf && P.near_stream && !P.serial;
     const bool dl = P.kernel == KIFMM_KERNEL_DL;
     // mixed DL: the FP32 remainders of the dipoles too (the near field's exact products)
     const bool dl_lo = dl && std::is_same<Real, float>::value;
@@ -3057,7 +3120,7 @@ extern "C" int kifmm_plan_get_stats(kifmm_plan plan, kifmm_plan_stats* st) {
     st->m2l_rows = P.fp64 ? P.Q : st->rank_down;
     st->near_units = P.n_p2p_units;
     st->near_split_leaves = P.n_p2p_split;
-    st->near_overlap = (!P.fp64 && P.near_stream && P.n_tleaf && warp_near(P)) ? 1 : 0;
+    st->near_overlap = (!P.fp64 && P.near_stream && P.n_tleaf) ? 1 : 0;
     st->near_corr_ranges = P.n_p2p_corr;
     st->near_axis_units = P.n_p2p_axis;
     st->near_pairs = P.near_pairs;

@@ -98,7 +98,9 @@ struct Plan {
     // work lists
     DBuf<int> s2u_box, s2u_off, s2u_idx;  // S2U: leaf boxes, CSR of source boxes (itself)
     DBuf<int> p2l_box, p2l_off, p2l_idx;  // X list: boxes, CSR of source leaves
-    DBuf<int> tleaf, p2p_off, p2p_idx;    // target leaves, CSR of U + W source boxes
+    DBuf<int> tleaf, p2p_off;             // target leaves, CSR offsets of their U + W (leaf X) source boxes
+    DBuf<longlong2> p2p_lranges;          // block kernel: the source ranges of that CSR
+    DBuf<int> p2p_order;                  //   and its leaves, heaviest first
     DBuf<int4> p2p_units;                 // mixed: near-field work units (leaf, first range,
                                           // end range, flags: 1 first of its leaf, 2 leaf split)
     DBuf<longlong2> p2p_ranges;           // mixed: source index ranges of the units
