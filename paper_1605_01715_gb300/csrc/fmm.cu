@@ -542,50 +542,72 @@ __global__ void __launch_bounds__(128) k_center(int box0, int Q, int Qp, Real* _
 }
 
 // ---------------------------------------------------------------- D2T
-// res[t] = T[t] . d[leaf(t)]: one block per target leaf, one warp per target row.
+// res[t] = T[t] . d[leaf(t)]: one block per target leaf, two rows at a time per warp (the
+// rows stream from HBM once; a small tree's few warps have two rows in flight each; four
+// lost 3 % on the 1M cube to leaves that are not a multiple of 16 rows).
 template <typename Real>
 __global__ void __launch_bounds__(128)
 k_d2t(const int* __restrict__ leaves, const int64_t* __restrict__ rng, const Real* __restrict__ T,
       const Real* __restrict__ d, int Qp, Real* __restrict__ res) {
-    extern __shared__ unsigned char smem_raw[];
+    constexpr int R = 2;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
     Real* ds = reinterpret_cast<Real*>(smem_raw);
     int b = leaves[blockIdx.x];
     for (int k = threadIdx.x; k < Qp; k += blockDim.x) ds[k] = d[(size_t)b * Qp + k];
     __syncthreads();
     int64_t tb = rng[4 * b + 2], te = rng[4 * b + 3];
     int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-    if constexpr (std::is_same<Real, float>::value) {
-        // FP32 rows (Qp a multiple of 16): 16-byte streaming loads, read once
-        const float4* ds4 = reinterpret_cast<const float4*>(ds);
-        for (int64_t t = tb + warp; t < te; t += blockDim.x / 32) {
-            const float4* row = reinterpret_cast<const float4*>(T + (size_t)t * Qp);
-            float s = 0.f;
+    for (int64_t t = tb + R * warp; t < te; t += R * (blockDim.x / 32)) {
+        const Real* row[R];
+        Real s[R];
+#pragma unroll
+        for (int u = 0; u < R; ++u) {
+            row[u] = T + (size_t)(t + u < te ? t + u : t) * Qp;
+            s[u] = 0;
+        }
+        if constexpr (std::is_same<Real, float>::value) {
+            // FP32 rows (Qp a multiple of 16): 16-byte streaming loads, read once
+            const float4* ds4 = reinterpret_cast<const float4*>(ds);
 #pragma unroll 2
             for (int k = lane; k < Qp / 4; k += 32) {
-                const float4 a = __ldcs(row + k), c = ds4[k];
-                s = fmaf(a.x, c.x, fmaf(a.y, c.y, fmaf(a.z, c.z, fmaf(a.w, c.w, s))));
+                const float4 c = ds4[k];
+                float4 a[R];
+#pragma unroll
+                for (int u = 0; u < R; ++u) a[u] = __ldcs(reinterpret_cast<const float4*>(row[u]) + k);
+#pragma unroll
+                for (int u = 0; u < R; ++u)
+                    s[u] = fmaf(a[u].x, c.x, fmaf(a[u].y, c.y, fmaf(a[u].z, c.z, fmaf(a[u].w, c.w, s[u]))));
             }
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (lane == 0) res[t] = s;
-        }
-    } else {
-        for (int64_t t = tb + warp; t < te; t += blockDim.x / 32) {
-            const Real* row = T + (size_t)t * Qp;
-            Real s = 0;
-            for (int k = lane; k < Qp; k += 32) s += row[k] * ds[k];
+        for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (lane == 0) res[t] = s;
+            for (int u = 0; u < R; ++u) s[u] += __shfl_xor_sync(0xffffffffu, s[u], o);
+#pragma unroll
+        for (int u = 0; u < R; ++u)
+            if (lane == u && t + u < te) res[t + u] = s[u];
+        } else {
+            for (int k = lane; k < Qp; k += 32) {
+                const Real c = ds[k];
+#pragma unroll
+                for (int u = 0; u < R; ++u) s[u] += __ldcs(row[u] + k) * c;
+            }
         }
     }
 }
 
 // ---------------------------------------------------------------- P2P (U and W lists) + scatter
-// One block per target leaf, one thread per target; source boxes staged in shared
-// memory relative to the target leaf's centre.
+// One block per target leaf, heaviest leaves first, one thread per target; a thread sums
+// over the leaf's sources in their list order.  Chunks of sources (as many as the block
+// has working threads) run across the leaf's source ranges and are staged relative to the
+// leaf's centre, double-buffered: the next chunk's coordinates are on their way to
+// registers while one is evaluated, and a chunk costs one barrier.  Warps without a target
+// leave at once.  What bounds it is the heaviest leaf (tens of thousands of W-list sources
+// in adaptive trees), whose chunks run one after the other.
 // KIND 0: q/r   1: (q n_j).(x - y)/r^3   2: q n_i.(x - y)/r^3   3: q (x - y)/r^3 (three
-// components, written to out[tperm[t] + c nt] with the far field res[t + c nt])
+// components, written to out[tperm[t] + c nt] with the far field res[t + c nt], if any)
+template <typename Real> struct Vec4;
+template <> struct Vec4<float> { using T = float4; using T2 = float2; };
+template <> struct Vec4<double> { using T = double4_32a; using T2 = double2; };
 template <typename Real, int KIND>
 __global__ void k_p2p(const int* __restrict__ order, const int* __restrict__ leaves, const int* __restrict__ off,
                       const longlong2* __restrict__ ranges, const int64_t* __restrict__ rng,
@@ -648,32 +670,6 @@ __global__ void k_p2p(const int* __restrict__ order, const int* __restrict__ lea
                     g2 = qs[2 * ns + j];
                 }
             }
-        }
-        if (valid) {
-            out[tperm[t]] = (double)(res ? acc + res[t] : acc);
-            if (KIND == 3) {
-                out[tperm[t] + nt] = (double)(res ? acc2 + res[t + nt] : acc2);
-                out[tperm[t] + 2 * nt] = (double)(res ? acc3 + res[t + 2 * nt] : acc3);
-            }
-        }
-    }
-}
-
-// FP32 near field (mixed form), one warp per work unit.  A unit is at most kP2PUnitSrc
-// sources of one target leaf (pieces of its U-, W- and X-list source ranges); units run
-// heaviest first, and a leaf spread over several units adds into its zeroed outputs
-// with FP64 atomics (the first unit also adds the far field).  Lanes form 4 source
-// groups of 8: lane (g, r) holds targets t0 + 8 i + r (i < T) of the current pass of
-// at most 8 T targets, packed in pairs so that every step is one FP32x2 instruction for
-// two pair evaluations, and takes sources g, g + 4, ... of each chunk of 32; the four
-// partial sums of a target meet by shuffles at the end.
-//
-// Chunks are double-buffered: while one chunk is evaluated, cp.async copies the next
-// chunk's raw source data (FP32 hi/lo coordinates and densities or dipoles) into shared
-// memory; each lane then turns its source into the staged form the pair loop reads by
-// shared-memory broadcast, every value already duplicated as a float2 pair.
-//
-// Accuracy (Sec. III.A.1 asks for the discrete sum; these are the steps that keep the
             return got;
         };
         auto term = [&](const R4& y, const R2* yd, Real& dx, Real& dy, Real& dz, Real& w, Real& v) {
