@@ -308,8 +308,9 @@ __device__ __forceinline__ void surf_pairs_ax(int ax, const float4* __restrict__
 //
 // A block holds the whole check potential of its box, so it also writes the box's input
 // for the tensor-core projection that follows: the potential scaled by the power of two
-// that puts its largest entry into [2^14, 2^15) (exponent in bexp[b]) and split into
-// FP16 hi and lo terms (Qp per box, zero past Q) -- the box split done in the producer.
+// that puts its largest entry into [2^14, 2^15) (exponent in bexp) and split into FP16 hi
+// and lo terms (Qp per box, zero past Q) -- the box split done in the producer.  S2U stores
+// them by box, the X list (down) by position in its list, in buffers of its own.
 // DIFF: the X list of a gradient kernel -- each check potential less the sources'
 // potential at the box centre (see surf_pairs), so that FP32 and the split keep the
 // variation across a box far smaller than its distance to the sources.
@@ -319,6 +320,7 @@ k_surf_f(const int* __restrict__ boxes, const int* __restrict__ off, const int* 
          const float4* __restrict__ bcf, const int64_t* __restrict__ rng, const float* __restrict__ sxf, int64_t ns,
          const float* __restrict__ qs, const float* __restrict__ surf, int Q, int Qp, __half* __restrict__ vin_h,
          __half* __restrict__ vin_l, int* __restrict__ bexp, const int* __restrict__ bax) {
+    const int slot = down ? (int)blockIdx.x : boxes[blockIdx.x];   // X boxes are stored in list order
     __shared__ float4 sp[NT];
     __shared__ float4 sd[(DIPOLE || DIFF) ? NT : 1];
     const int b = boxes[blockIdx.x];
@@ -418,10 +420,10 @@ k_surf_f(const int* __restrict__ boxes, const int* __restrict__ off, const int* 
     for (int w = 1; w < NT / 32; ++w) mx = fmaxf(mx, s_red[w]);
     int ex = mx > 0.f ? 14 - ilogbf(mx) : 0;
     ex = max(-100, min(100, ex));
-    if (threadIdx.x == 0) bexp[b] = ex;
+    if (threadIdx.x == 0) bexp[slot] = ex;
     const float sc = __int_as_float((127 + ex) << 23);
-    __half* hb = vin_h + (size_t)b * Qp;
-    __half* lb = vin_l + (size_t)b * Qp;
+    __half* hb = vin_h + (size_t)slot * Qp;
+    __half* lb = vin_l + (size_t)slot * Qp;
 #pragma unroll
     for (int m = 0; m < NP; ++m) {
 #pragma unroll
@@ -485,20 +487,22 @@ int launch_surf(const Plan& P, const Tree& T, bool dl, int nbox, const int* boxe
         const float* sf = down ? P.surf_f.p : P.ops->surf_up.p;
         const int slots = down ? surf_slots_full(P.Q) : surf_slots(npts);
         const bool diff = down && !dl && gradient_kernel(P.kernel);
+        __half* oh = down ? P.xin_h.p : P.sin_h.p;
+        __half* ol = down ? P.xin_l.p : P.sin_l.p;
+        int* oe = down ? P.xexp.p : P.sexp.p;
         switch (slots * 2 + (dl ? 1 : 0)) {
 #define KF_SURF(NP, NT)                                                                                          \
     case 2 * (2 * NP * NT):                                                                                      \
         if (diff)                                                                                                \
             k_surf_f<false, NP, NT, true><<<nbox, NT, 0, s>>>(boxes, off, idx, down, P.bcf.p, T.rng.p, P.sxf.p,  \
-                                                              T.ns, q, sf, npts, stride, P.sin_h.p, P.sin_l.p,   \
-                                                              P.sexp.p, nullptr);                                \
+                                                              T.ns, q, sf, npts, stride, oh, ol, oe, nullptr);    \
         else                                                                                                     \
             k_surf_f<false, NP, NT><<<nbox, NT, 0, s>>>(boxes, off, idx, down, P.bcf.p, T.rng.p, P.sxf.p, T.ns, q,  \
-                                                        sf, npts, stride, P.sin_h.p, P.sin_l.p, P.sexp.p, nullptr); \
+                                                        sf, npts, stride, oh, ol, oe, nullptr);             \
         break;                                                                                                   \
     case 2 * (2 * NP * NT) + 1:                                                                                  \
         k_surf_f<true, NP, NT><<<nbox, NT, 0, s>>>(boxes, off, idx, down, P.bcf.p, T.rng.p, P.sxf.p, T.ns, q, sf,    \
-                                                   npts, stride, P.sin_h.p, P.sin_l.p, P.sexp.p, P.bax.p);       \
+                                                   npts, stride, oh, ol, oe, P.bax.p);                 \
         break;
             KF_SURF(1, 128) KF_SURF(2, 96) KF_SURF(2, 128) KF_SURF(3, 96) KF_SURF(3, 128) KF_SURF(4, 128)
 #undef KF_SURF
@@ -578,13 +582,6 @@ k_d2t(const int* __restrict__ leaves, const int64_t* __restrict__ rng, const Rea
                 for (int u = 0; u < R; ++u)
                     s[u] = fmaf(a[u].x, c.x, fmaf(a[u].y, c.y, fmaf(a[u].z, c.z, fmaf(a[u].w, c.w, s[u]))));
             }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-            for (int u = 0; u < R; ++u) s[u] += __shfl_xor_sync(0xffffffffu, s[u], o);
-#pragma unroll
-        for (int u = 0; u < R; ++u)
-            if (lane == u && t + u < te) res[t + u] = s[u];
         } else {
             for (int k = lane; k < Qp; k += 32) {
                 const Real c = ds[k];
@@ -592,6 +589,13 @@ k_d2t(const int* __restrict__ leaves, const int64_t* __restrict__ rng, const Rea
                 for (int u = 0; u < R; ++u) s[u] += __ldcs(row[u] + k) * c;
             }
         }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int u = 0; u < R; ++u) s[u] += __shfl_xor_sync(0xffffffffu, s[u], o);
+#pragma unroll
+        for (int u = 0; u < R; ++u)
+            if (lane == u && t + u < te) res[t + u] = s[u];
     }
 }
 
@@ -722,9 +726,35 @@ __global__ void k_p2p(const int* __restrict__ order, const int* __restrict__ lea
             }
             buf ^= 1;
             cnt = ncnt;
-// FP32 evaluation at the single layer's accuracy for all three kernels):
+        }
         // the last chunk is read before the next pass stages its first
         asm volatile("bar.sync 1, %0;" ::"r"(nthr) : "memory");
+        if (valid) {
+            out[tperm[t]] = (double)(res ? acc + res[t] : acc);
+            if (KIND == 3) {
+                out[tperm[t] + nt] = (double)(res ? acc2 + res[t + nt] : acc2);
+                out[tperm[t] + 2 * nt] = (double)(res ? acc3 + res[t + 2 * nt] : acc3);
+            }
+        }
+    }
+}
+
+// FP32 near field (mixed form), one warp per work unit.  A unit is at most kP2PUnitSrc
+// sources of one target leaf (pieces of its U-, W- and X-list source ranges); units run
+// heaviest first, and a leaf spread over several units adds into its zeroed outputs
+// with FP64 atomics (the first unit also adds the far field).  Lanes form 4 source
+// groups of 8: lane (g, r) holds targets t0 + 8 i + r (i < T) of the current pass of
+// at most 8 T targets, packed in pairs so that every step is one FP32x2 instruction for
+// two pair evaluations, and takes sources g, g + 4, ... of each chunk of 32; the four
+// partial sums of a target meet by shuffles at the end.
+//
+// Chunks are double-buffered: while one chunk is evaluated, cp.async copies the next
+// chunk's raw source data (FP32 hi/lo coordinates and densities or dipoles) into shared
+// memory; each lane then turns its source into the staged form the pair loop reads by
+// shared-memory broadcast, every value already duplicated as a float2 pair.
+//
+// Accuracy (Sec. III.A.1 asks for the discrete sum; these are the steps that keep the
+// FP32 evaluation at the single layer's accuracy for all three kernels):
 //  - Offsets are taken from the leaf centre.  Each range has an exponent E with every
 //    coordinate offset of the leaf's targets and the range's sources below 2^E (from
 //    the boxes' extents).  For the double layers an offset is split as hi + lo, hi on the
@@ -2476,16 +2506,26 @@ int setup(Plan& P, const double* src_nrm, const double* trg_nrm, cudaStream_t s)
             std::vector<int4> tiles;
             std::vector<int> pin, pout;
             std::vector<Triple> tr;
-            for (int b : up ? s2u_box : p2l_box) tr.push_back({0, b, b});
+            if (up)
+                for (int b : s2u_box) tr.push_back({0, b, b});
+            else
+                for (int i = 0; i < P.n_p2l; ++i) tr.push_back({0, i, p2l_box[i]});
             make_tiles(tr, tiles, pin, pout, cap_for(tr, up ? cap_up : cap_dn, up ? P.ops->Ku : P.ops->Kd));
             KF_TRY(upload_tiles(up ? P.proj_up : P.proj_x, tiles, pin, pout, s));
         }
+        KF_TRY(P.xexp.alloc(P.n_p2l));
+        KF_TRY(P.xin_h.alloc((size_t)P.n_p2l * P.Qp));
+        KF_TRY(P.xin_l.alloc((size_t)P.n_p2l * P.Qp));
         KF_TRY(P.zu.alloc((size_t)T.nbox * P.ops->Ku));
         KF_TRY(P.zd.alloc((size_t)T.nbox * P.ops->Kd));
         int prio_lo = 0, prio_hi = 0;
         KF_CHECK_CUDA(cudaDeviceGetStreamPriorityRange(&prio_lo, &prio_hi));
         KF_CHECK_CUDA(cudaStreamCreateWithPriority(&P.near_stream, cudaStreamNonBlocking, prio_lo));
         KF_CHECK_CUDA(cudaStreamCreateWithPriority(&P.far_stream, cudaStreamNonBlocking, prio_hi));
+        if (P.n_p2l) {
+            KF_CHECK_CUDA(cudaStreamCreateWithPriority(&P.x_stream, cudaStreamNonBlocking, prio_hi));
+            KF_CHECK_CUDA(cudaEventCreateWithFlags(&P.ev_x, cudaEventDisableTiming));
+        }
         KF_CHECK_CUDA(cudaEventCreateWithFlags(&P.ev_fork, cudaEventDisableTiming));
         KF_CHECK_CUDA(cudaEventCreateWithFlags(&P.ev_join, cudaEventDisableTiming));
         KF_CHECK_CUDA(cudaEventCreateWithFlags(&P.ev_far, cudaEventDisableTiming));
@@ -2531,7 +2571,7 @@ int setup(Plan& P, const double* src_nrm, const double* trg_nrm, cudaStream_t s)
                      P.res_d.bytes(), P.q_d.bytes(), P.u_f.bytes(), P.d_f.bytes(), P.res_f.bytes(),
                      P.q_f.bytes(), P.snrm.bytes(), P.tnrm_d.bytes(), P.tnrm_f.bytes(),
                      P.bexp.bytes(), P.vsl.bytes(), P.vin_h.bytes(), P.vin_l.bytes(), P.sexp.bytes(), P.sin_h.bytes(),
-                     P.sin_l.bytes(), P.sxf.bytes(), P.txf.bytes(), P.bcf.bytes(), P.zu.bytes(),
+                     P.sin_l.bytes(), P.xexp.bytes(), P.xin_h.bytes(), P.xin_l.bytes(), P.sxf.bytes(), P.txf.bytes(), P.bcf.bytes(), P.zu.bytes(),
                      P.zd.bytes()})
         P.device_bytes += (int64_t)b;
     return KIFMM_OK;
@@ -2553,6 +2593,8 @@ int run_pairs(const Plan& P, int which, const PairTiles& pt, int t0, int t1, con
 // (the 1M cube at 128 points per leaf: 52, once its exact zeros are left out; at 192:
 // 298; curved surfaces: several hundred).
 constexpr int64_t kLateNearPairs = 100;
+// Near-field pairs from which the X list stays in the far field's chain.
+constexpr int64_t kXBesidePairs = 300000000;
 
 // Mixed precision: two-term FP16 on the tensor cores (tcgen05), every translation
 // between projected check potentials (see build_projected): U2U in the up basis (ru of
@@ -2592,14 +2634,16 @@ int run_pairs<float>(const Plan& P, int which, const PairTiles& pt, int t0, int 
 
 // Mixed: projection of the full check potentials of the boxes in pt's tiles onto the up
 // (fam 3) or down (fam 4) basis, added into z.  Their split inputs (sin_h/sin_l, Qp per
-// box, exponents in sexp) were written by the surface kernel that computed them.
+// box, exponents in sexp; the X list's in xin_h/xin_l, xexp) were written by the surface
+// kernel that computed them.
 int project(const Plan& P, int fam, const PairTiles& pt, float* z, cudaStream_t s, int& launches) {
     if (pt.ntiles == 0) return KIFMM_OK;
     const OpTables& o = *P.ops;
     const int Mr = fam == 3 ? o.Ku : o.Kd, M = fam == 3 ? o.ru : o.rd, Kp = fam == 3 ? o.ks : P.Qp;
     const CUtensorMap* m = o.tmaps[fam];
-    KF_TRY(launch_pair_tc(3, m[0], m[1], o.texp[fam], M, Mr, Kp, Mr, pt.tiles.p, pt.ntiles, pt.pin.p,
-                          pt.pout.p, P.sexp.p, P.sin_h.p, P.sin_l.p, z, P.err.p, s));
+    KF_TRY(launch_pair_tc(3, m[0], m[1], o.texp[fam], M, Mr, Kp, Mr, pt.tiles.p, pt.ntiles, pt.pin.p, pt.pout.p,
+                          fam == 3 ? P.sexp.p : P.xexp.p, fam == 3 ? P.sin_h.p : P.xin_h.p,
+                          fam == 3 ? P.sin_l.p : P.xin_l.p, z, P.err.p, s));
     launches += 2;
     return KIFMM_OK;
 }
@@ -2773,6 +2817,23 @@ int matvec(Plan& P, const Bufs<Real>& B, const double* q, double* out, cudaStrea
         }
         ++launches;
     }
+    // The X list needs only the gathered sources: beside the upward pass and M2L, on a stream
+    // of its own that joins the far field before L2L (both add into zd by atomics): in
+    // series it was 72 of the 280 us of an 8-sphere polarization step, 17 of 166 of the 20k
+    // sphere.  A large near field fills the SMs by itself, and then the X list only delays it
+    // (64-sphere pack, 628M near pairs: 1956 in series, 1984 us beside).
+    const bool x_overlap = mixed && near_overlap && P.n_p2l > 0 && P.near_pairs < kXBesidePairs;
+    if constexpr (mixed) {
+        if (x_overlap) {
+            KF_CHECK_CUDA(cudaStreamWaitEvent(P.x_stream, P.ev_fork, 0));
+            KF_TRY(launch_surf<Real>(P, T, dl, P.n_p2l, P.p2l_box.p, P.p2l_off.p, P.p2l_idx.p, kDnCheck, B.q, B.surf, B.d,
+                                     P.x_stream));
+            ++launches;
+            KF_CHECK_CUDA(cudaStreamWaitEvent(P.x_stream, P.ev_zero, 0));
+            KF_TRY(project(P, 4, P.proj_x, dn, P.x_stream, launches));
+            KF_CHECK_CUDA(cudaEventRecord(P.ev_x, P.x_stream));
+        }
+    }
     // A near field much smaller than the far field (few evaluated pairs per target, as on
     // flat faces) starts after M2L, beside the coarse L2L levels and D2T, rather than
     // beside S2U and the upward pass, whose arithmetic it would slow.
@@ -2790,7 +2851,7 @@ int matvec(Plan& P, const Bufs<Real>& B, const double* q, double* out, cudaStrea
                                launches));
     KF_TRY(mark(3));
     // X list (mixed: then the X boxes' projections), then V list
-    if (P.n_p2l) {
+    if (P.n_p2l && !x_overlap) {
         // (the Chebyshev engine: X sources straight onto the box's nodes)
         KF_TRY(launch_surf<Real>(P, T, dl, P.n_p2l, P.p2l_box.p, P.p2l_off.p, P.p2l_idx.p, P.cheb ? 1.0 : kDnCheck,
                                  B.q, B.surf, B.d, s));
@@ -2805,6 +2866,7 @@ int matvec(Plan& P, const Bufs<Real>& B, const double* q, double* out, cudaStrea
         KF_CHECK_CUDA(cudaEventRecord(P.ev_fork, s));
         KF_TRY(fork_near());
     }
+    if (x_overlap) KF_CHECK_CUDA(cudaStreamWaitEvent(s, P.ev_x, 0));
     KF_TRY(mark(5));
     // L2L, coarsest children first (ADL in FP64: each level's potentials shifted to zero
     // mean first; the mixed tables carry that centring)

@@ -83,6 +83,8 @@ struct Plan {
     DBuf<float> d2t_f;
     DBuf<int> bexp, sexp;
     DBuf<__half> vin_h, vin_l, sin_h, sin_l;
+    DBuf<int> xexp;                 // mixed: the same of the X list, by position in it (it runs beside S2U)
+    DBuf<__half> xin_h, xin_l;
     DBuf<__half> vsl;               // FP64: the check potentials a translation reads, sliced (exponents in bexp)
     DBuf<double> surf_d;            // Q x 3 unit surface
     DBuf<float> surf_f;
@@ -148,6 +150,8 @@ struct Plan {
     // far field's many short launches leave idle; both join the caller's stream before
     // the far-field sum is added
     cudaStream_t near_stream = nullptr, far_stream = nullptr;
+    cudaStream_t x_stream = nullptr;   // the X list, beside the upward pass and M2L
+    cudaEvent_t ev_x = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_far = nullptr, ev_zero = nullptr;
     const double* g_q = nullptr;
     double* g_out = nullptr;
@@ -177,6 +181,8 @@ struct Plan {
         if (ev_join) cudaEventDestroy(ev_join);
         if (ev_far) cudaEventDestroy(ev_far);
         if (ev_zero) cudaEventDestroy(ev_zero);
+        if (ev_x) cudaEventDestroy(ev_x);
+        if (x_stream) cudaStreamDestroy(x_stream);
         if (near_stream) cudaStreamDestroy(near_stream);
         if (far_stream) cudaStreamDestroy(far_stream);
     }
