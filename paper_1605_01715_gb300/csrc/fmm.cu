@@ -554,7 +554,7 @@ __global__ void __launch_bounds__(128)
 k_d2t(const int* __restrict__ leaves, const int64_t* __restrict__ rng, const Real* __restrict__ T,
       const Real* __restrict__ d, int Qp, Real* __restrict__ res) {
     constexpr int R = 2;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
+    extern __shared__ __align__(32) unsigned char smem_raw[];
     Real* ds = reinterpret_cast<Real*>(smem_raw);
     int b = leaves[blockIdx.x];
     for (int k = threadIdx.x; k < Qp; k += blockDim.x) ds[k] = d[(size_t)b * Qp + k];
@@ -1280,26 +1280,51 @@ inline bool warp_near(const Plan& P) {
 // target leaf leaves[rleaf[i]]), the smallest FP64 squared distance between one of the
 // leaf's targets and one of the range's sources, over all pairs (minr2[2i]) and over the
 // pairs at least delta/2 apart (minr2[2i + 1]; coincident points, a target among its own
-// sources above all, are skipped whatever the precision).  One warp per range.
+// sources above all, are skipped whatever the precision), as far as it is below the
+// thresholds the ranges are flagged by: only pairs whose FP32 distance is within twice the
+// larger of 2^(E - kCloseBits) and 4 delta are evaluated in FP64.  (FP32 offsets are good to
+// 2^-22 of 2^E, 2^-17 of that threshold.  In FP64 throughout, the scan of 98,000 points took
+// 1.96 ms at the FP64 pipe's rate.)  One warp per range.
 __global__ void k_range_min_r2(int nr, const longlong2* __restrict__ ranges, const int* __restrict__ rleaf,
                                const int* __restrict__ leaves, const int64_t* __restrict__ rng,
-                               const double* __restrict__ sxyz, int64_t ns, const double* __restrict__ txyz,
-                               int64_t nt, double* __restrict__ minr2) {
+                               const float4* __restrict__ bcf, const float* __restrict__ sxf,
+                               const float* __restrict__ txf, const double* __restrict__ sxyz, int64_t ns,
+                               const double* __restrict__ txyz, int64_t nt, double* __restrict__ minr2) {
     const int i = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
     const int lane = threadIdx.x & 31;
     if (i >= nr) return;
     const int64_t j0 = ranges[i].x & kRangeIdx, j1 = ranges[i].y;
     const int b = leaves[rleaf[i]];
     const int64_t tb = rng[4 * b + 2], te = rng[4 * b + 3];
+    const float4 ch = bcf[3 * b], cl = bcf[3 * b + 1];
+    const float thr = 2.f * fmaxf(exp2i(range_exp(ranges[i].x) - kCloseBits), (float)(4.0 * kDelta));
+    const float thr2 = thr * thr;
     const double half2 = 0.25 * kDelta * kDelta;
     double best = 1e300, best_far = 1e300;
-    for (int64_t j = j0 + lane; j < j1; j += 32) {
-        const double sx = sxyz[j], sy = sxyz[ns + j], sz = sxyz[2 * ns + j];
-        for (int64_t t = tb; t < te; ++t) {
-            const double dx = txyz[t] - sx, dy = txyz[nt + t] - sy, dz = txyz[2 * nt + t] - sz;
-            const double r2 = dx * dx + dy * dy + dz * dz;
-            best = fmin(best, r2);
-            if (r2 >= half2) best_far = fmin(best_far, r2);
+    // a warp takes 32 sources; each lane's target offset is passed round by shuffles
+    for (int64_t jb = j0; jb < j1; jb += 32) {
+        const int64_t j = jb + lane;
+        const bool in = j < j1;
+        const int64_t jj = in ? j : j0;
+        const float sx = (sxf[jj] - ch.x) + (sxf[3 * ns + jj] - cl.x), sy = (sxf[ns + jj] - ch.y) + (sxf[4 * ns + jj] - cl.y),
+                    sz = (sxf[2 * ns + jj] - ch.z) + (sxf[5 * ns + jj] - cl.z);
+        for (int64_t t0 = tb; t0 < te; t0 += 32) {
+            const int64_t tt = t0 + lane < te ? t0 + lane : tb;
+            const float tx = (txf[tt] - ch.x) + (txf[3 * nt + tt] - cl.x), ty = (txf[nt + tt] - ch.y) + (txf[4 * nt + tt] - cl.y),
+                        tz = (txf[2 * nt + tt] - ch.z) + (txf[5 * nt + tt] - cl.z);
+            const int n = (int)(te - t0 < 32 ? te - t0 : 32);
+            for (int u = 0; u < n; ++u) {
+                const float ax = __shfl_sync(0xffffffffu, tx, u) - sx, ay = __shfl_sync(0xffffffffu, ty, u) - sy,
+                            az = __shfl_sync(0xffffffffu, tz, u) - sz;
+                if (in && !(ax * ax + ay * ay + az * az > thr2)) {
+                    const int64_t t = t0 + u;
+                    const double dx = txyz[t] - sxyz[j], dy = txyz[nt + t] - sxyz[ns + j], dz = txyz[2 * nt + t] - sxyz[2 * ns + j];
+                    const double r2 = dx * dx + dy * dy + dz * dz;
+                    best = fmin(best, r2);
+                    if (r2 >= half2) best_far = fmin(best_far, r2);
+                }
+                __syncwarp();
+            }
         }
     }
 #pragma unroll
@@ -1476,17 +1501,24 @@ void m2l_schedule(std::vector<Triple>& tr, const std::vector<int>& level, int ca
     auto by_out_op = [](const Triple& a, const Triple& b) { return a.out != b.out ? a.out < b.out : a.op < b.op; };
     bool grouped = true;
     for (size_t i = 1; i < tr.size() && grouped; ++i) grouped = tr[i - 1].out <= tr[i].out;
-    if (grouped) {
-        for (size_t i = 0; i < tr.size();) {
-            size_t j = i;
-            while (j < tr.size() && tr[j].out == tr[i].out) ++j;
-            std::stable_sort(tr.begin() + i, tr.begin() + j, by_out_op);
-            i = j;
-        }
-    } else {
-        std::stable_sort(tr.begin(), tr.end(), by_out_op);
+    if (!grouped) std::stable_sort(tr.begin(), tr.end(), by_out_op);
+    std::vector<size_t> beg;                          // each target's first triple, and the end
+    for (size_t i = 0; i < tr.size(); ++i)
+        if (i == 0 || tr[i].out != tr[i - 1].out) beg.push_back(i);
+    beg.push_back(tr.size());
+    // a hash of each target's (level, offsets); only targets whose hash many share can chain
+    std::vector<uint64_t> hash(beg.size() - 1);
+#pragma omp parallel for schedule(static)
+    for (int64_t q = 0; q < (int64_t)hash.size(); ++q) {
+        std::stable_sort(tr.begin() + beg[q], tr.begin() + beg[q + 1], by_out_op);
+        uint64_t h = 1469598103934665603ull ^ (uint64_t)(uint32_t)level[tr[beg[q]].out];
+        for (size_t i = beg[q]; i < beg[q + 1]; ++i) h = (h ^ (uint64_t)(uint32_t)tr[i].op) * 1099511628211ull;
+        hash[q] = h;
     }
-    // targets by (level, offsets of the V list), members in box order; groups are
+    std::unordered_map<uint64_t, size_t> nsame;
+    nsame.reserve(2 * hash.size());
+    for (uint64_t h : hash) ++nsame[h];
+    // those targets by (level, offsets of the V list), members in box order; groups are
     // visited in the order of their (level, offsets) keys
     struct KeyHash {
         size_t operator()(const std::pair<int, std::vector<int>>& k) const {
@@ -1496,12 +1528,11 @@ void m2l_schedule(std::vector<Triple>& tr, const std::vector<int>& level, int ca
         }
     };
     std::unordered_map<std::pair<int, std::vector<int>>, std::vector<std::pair<int, size_t>>, KeyHash> hgroups;
-    for (size_t i = 0; i < tr.size();) {
-        size_t j = i;
+    for (size_t q = 0; q < hash.size(); ++q) {
+        if (nsame[hash[q]] * 4 < (size_t)cap * 3) continue;
         std::vector<int> sig;
-        while (j < tr.size() && tr[j].out == tr[i].out) sig.push_back(tr[j++].op);
-        hgroups[{level[tr[i].out], std::move(sig)}].push_back({tr[i].out, i});
-        i = j;
+        for (size_t i = beg[q]; i < beg[q + 1]; ++i) sig.push_back(tr[i].op);
+        hgroups[{level[tr[beg[q]].out], std::move(sig)}].push_back({tr[beg[q]].out, beg[q]});
     }
     std::vector<const std::pair<const std::pair<int, std::vector<int>>, std::vector<std::pair<int, size_t>>>*> groups;
     groups.reserve(hgroups.size());
@@ -2163,6 +2194,14 @@ int setup(Plan& P, const double* src_nrm, const double* trg_nrm, cudaStream_t s)
             if (tx[(size_t)k * ntp + q] != c) return false;
         return true;
     };
+    // every box's axis and plane, each box by one thread (read-only from here on)
+    if (!plane_k.empty()) {
+#pragma omp parallel for schedule(dynamic, 256)
+        for (int b = 0; b < T.nbox; ++b) {
+            axis_class(b);
+            src_plane(b);
+        }
+    }
     for (int b = 0; b < T.nbox; ++b) {
         int l = T.h_lvl[b];
         if (T.h_leaf[b] && has_src(T, b) && l >= 2) {
@@ -2252,69 +2291,86 @@ int setup(Plan& P, const double* src_nrm, const double* trg_nrm, cudaStream_t s)
         std::vector<Unit> units;
         std::vector<longlong2> ranges;
         std::vector<int> rleaf;
-        std::vector<double> rext;              // per range: largest coordinate offset of its pairs
+        std::vector<signed char> ucls;         // DL: the dipole axis class of a unit's boxes
         auto half = [&](int box) { return std::ldexp(T.root_h, -T.h_lvl[box]); };
         auto exp_of = [](double ext) { return std::max(-100, std::min(100, std::ilogb(ext * (1.0 + 1e-12)) + 1)); };
-        std::vector<int> lb;
-        for (size_t li = 0; li < tleaf.size(); ++li) {
-            const int b = tleaf[li];
-            const int64_t ntg = T.h_rng[4 * b + 3] - T.h_rng[4 * b + 2];
-            const double hb = half(b);
-            const size_t u0 = units.size();
-            int r0 = (int)ranges.size();
-            int64_t cnt = 0;
-            auto close_unit = [&]() {
-                // order the unit's ranges by exponent
-                std::vector<int> ord(ranges.size() - r0);
-                std::iota(ord.begin(), ord.end(), r0);
-                std::stable_sort(ord.begin(), ord.end(), [&](int x, int y) {
-                    return range_exp(ranges[x].x) < range_exp(ranges[y].x);
-                });
-                std::vector<longlong2> rg;
-                std::vector<double> re;
-                for (int i : ord) {
-                    rg.push_back(ranges[i]);
-                    re.push_back(rext[i]);
+        // leaves are independent: blocks of them by thread, joined in leaf order
+        constexpr size_t kLeafBlock = 128;
+        const size_t nblk = (tleaf.size() + kLeafBlock - 1) / kLeafBlock;
+        struct Block {
+            std::vector<Unit> units;
+            std::vector<longlong2> ranges;
+            std::vector<int> rleaf;
+            std::vector<signed char> ucls;
+            int split = 0;
+        };
+        std::vector<Block> blocks(nblk);
+#pragma omp parallel for schedule(dynamic, 1)
+        for (int64_t bi = 0; bi < (int64_t)nblk; ++bi) {
+            Block& B = blocks[bi];
+            std::vector<int> lb;
+            for (size_t li = bi * kLeafBlock; li < std::min(tleaf.size(), (size_t)(bi + 1) * kLeafBlock); ++li) {
+                const int b = tleaf[li];
+                const int64_t ntg = T.h_rng[4 * b + 3] - T.h_rng[4 * b + 2];
+                const double hb = half(b);
+                const size_t u0 = B.units.size();
+                int r0 = (int)B.ranges.size();
+                int64_t cnt = 0;
+                int cls_cur = -1;
+                auto close_unit = [&]() {
+                    // order the unit's ranges by exponent
+                    std::stable_sort(B.ranges.begin() + r0, B.ranges.end(), [](const longlong2& x, const longlong2& y) {
+                        return range_exp(x.x) < range_exp(y.x);
+                    });
+                    B.units.push_back({make_int4((int)li, r0, (int)B.ranges.size(), 0), ntg * cnt});
+                    B.ucls.push_back((signed char)cls_cur);
+                    r0 = (int)B.ranges.size();
+                    cnt = 0;
+                };
+                lb.assign(p2p_idx.begin() + p2p_off[li], p2p_idx.begin() + p2p_off[li + 1]);
+                if (!box_ax.empty())
+                    std::stable_sort(lb.begin(), lb.end(), [&](int x, int y) { return axis_class(x) < axis_class(y); });
+                for (const int a : lb) {
+                    const int cls = axis_class(a);
+                    if (cnt > 0 && cls != cls_cur) close_unit();
+                    cls_cur = cls;
+                    const double ha = half(a);
+                    double box_ext = hb;
+                    for (int d = 0; d < 3; ++d) {
+                        const double ca = (2 * T.h_coord[3 * a + d] + 1) * ha, cb = (2 * T.h_coord[3 * b + d] + 1) * hb;
+                        box_ext = std::max(box_ext, std::fabs(ca - cb) + ha);
+                    }
+                    const long long ebits = (long long)(exp_of(box_ext) + 128) << 48;
+                    int64_t j0 = T.h_rng[4 * a], j1 = T.h_rng[4 * a + 1];
+                    while (j0 < j1) {
+                        const int64_t take = std::min<int64_t>(j1 - j0, kP2PUnitSrc - cnt);
+                        B.ranges.push_back(make_longlong2(j0 | ebits, j0 + take));
+                        B.rleaf.push_back((int)li);
+                        cnt += take;
+                        j0 += take;
+                        if (cnt == kP2PUnitSrc) close_unit();
+                    }
                 }
-                std::copy(rg.begin(), rg.end(), ranges.begin() + r0);
-                std::copy(re.begin(), re.end(), rext.begin() + r0);
-                units.push_back({make_int4((int)li, r0, (int)ranges.size(), 0), ntg * cnt});
-                r0 = (int)ranges.size();
-                cnt = 0;
-            };
-            lb.assign(p2p_idx.begin() + p2p_off[li], p2p_idx.begin() + p2p_off[li + 1]);
-            if (!box_ax.empty())
-                std::stable_sort(lb.begin(), lb.end(), [&](int x, int y) { return axis_class(x) < axis_class(y); });
-            int cls_cur = -1;
-            for (const int a : lb) {
-                const int cls = axis_class(a);
-                if (cnt > 0 && cls != cls_cur) close_unit();
-                cls_cur = cls;
-                const double ha = half(a);
-                double box_ext = hb;
-                for (int d = 0; d < 3; ++d) {
-                    const double ca = (2 * T.h_coord[3 * a + d] + 1) * ha, cb = (2 * T.h_coord[3 * b + d] + 1) * hb;
-                    box_ext = std::max(box_ext, std::fabs(ca - cb) + ha);
-                }
-                const long long ebits = (long long)(exp_of(box_ext) + 128) << 48;
-                int64_t j0 = T.h_rng[4 * a], j1 = T.h_rng[4 * a + 1];
-                while (j0 < j1) {
-                    const int64_t take = std::min<int64_t>(j1 - j0, kP2PUnitSrc - cnt);
-                    ranges.push_back(make_longlong2(j0 | ebits, j0 + take));
-                    rleaf.push_back((int)li);
-                    rext.push_back(box_ext);
-                    cnt += take;
-                    j0 += take;
-                    if (cnt == kP2PUnitSrc) close_unit();
-                }
+                if (cnt > 0 || B.units.size() == u0) close_unit();
+                const bool split = B.units.size() - u0 > 1;
+                B.split += split ? 1 : 0;
+                for (size_t i = u0; i < B.units.size(); ++i)
+                    B.units[i].u.w = (i == u0 ? kUnitFirst : 0) | (split ? kUnitSplit : 0);
             }
-            if (cnt > 0 || units.size() == u0) close_unit();
-            const bool split = units.size() - u0 > 1;
-            P.p2p_multi = P.p2p_multi || split;
-            P.n_p2p_split += split ? 1 : 0;
-            for (size_t i = u0; i < units.size(); ++i)
-                units[i].u.w = (i == u0 ? kUnitFirst : 0) | (split ? kUnitSplit : 0);
         }
+        for (const Block& B : blocks) {
+            const int r0 = (int)ranges.size();
+            ranges.insert(ranges.end(), B.ranges.begin(), B.ranges.end());
+            rleaf.insert(rleaf.end(), B.rleaf.begin(), B.rleaf.end());
+            ucls.insert(ucls.end(), B.ucls.begin(), B.ucls.end());
+            for (Unit u : B.units) {
+                u.u.y += r0;
+                u.u.z += r0;
+                units.push_back(u);
+            }
+            P.n_p2p_split += B.split;
+        }
+        P.p2p_multi = P.n_p2p_split > 0;
         // FP64 scan: the closest pair of each range
         const int nr = (int)ranges.size();
         std::vector<int4> hcu;
@@ -2327,8 +2383,9 @@ int setup(Plan& P, const double* src_nrm, const double* trg_nrm, cudaStream_t s)
             KF_TRY(drl.upload(rleaf, s));
             KF_TRY(dmin.alloc(2 * (size_t)nr));
             const double* txyz = T.same ? T.sxyz.p : T.txyz.p;
-            k_range_min_r2<<<div_up((int64_t)nr * 32, 256), 256, 0, s>>>(nr, dr.p, drl.p, P.tleaf.p, T.rng.p, T.sxyz.p,
-                                                                       T.ns, txyz, T.nt, dmin.p);
+            k_range_min_r2<<<div_up((int64_t)nr * 32, 256), 256, 0, s>>>(nr, dr.p, drl.p, P.tleaf.p, T.rng.p, P.bcf.p,
+                                                                       P.sxf.p, T.same ? P.sxf.p : P.txf.p,
+                                                                       T.sxyz.p, T.ns, txyz, T.nt, dmin.p);
             KF_CHECK_LAUNCH();
             std::vector<double> minr2;
             KF_TRY(download(minr2, dmin.p, 2 * (size_t)nr, s));
@@ -2350,26 +2407,24 @@ int setup(Plan& P, const double* src_nrm, const double* trg_nrm, cudaStream_t s)
         // the one-term kernel (KIND 4), dealt after the others
         std::vector<char> is_axis(units.size(), 0);
         if (P.kernel == KIFMM_KERNEL_DL && T.ns > 0) {
-            std::vector<double> hn;
-            KF_TRY(download(hn, P.snrm.p, 3 * (size_t)T.ns, s));
-            std::vector<signed char> ax(T.ns);
-            for (int64_t j = 0; j < T.ns; ++j) {
-                const double c[3] = {hn[j], hn[T.ns + j], hn[2 * T.ns + j]};
-                ax[j] = -1;
-                for (int k = 0; k < 3; ++k)
-                    if (c[(k + 1) % 3] == 0.0 && c[(k + 2) % 3] == 0.0 && c[k] != 0.0) ax[j] = (signed char)k;
-            }
-            // run[j]: end of the run of equal axis codes from j
-            std::vector<int64_t> run(T.ns);
-            for (int64_t j = T.ns - 1; j >= 0; --j)
-                run[j] = (j + 1 < T.ns && ax[j + 1] == ax[j]) ? run[j + 1] : j + 1;
-            for (size_t i = 0; i < units.size(); ++i) {
-                int k = -2;
-                for (int r = units[i].u.y; r < units[i].u.z && k != -1; ++r) {
-                    const int64_t j0 = ranges[r].x & kRangeIdx, j1 = ranges[r].y;
-                    const int kr = (run[j0] >= j1) ? ax[j0] : -1;
-                    k = (k == -2 || k == kr) ? kr : -1;
-                }
+            // the axis of source j's dipole, or -1
+            auto axis_of = [&](int64_t j) {
+                int k = -1;
+                for (int d = 0; d < 3; ++d)
+                    if (hsn[(size_t)d * T.ns + j] != 0.0) k = k == -1 ? d : -2;
+                return k < 0 ? -1 : k;
+            };
+#pragma omp parallel for schedule(dynamic, 256)
+            for (int64_t i = 0; i < (int64_t)units.size(); ++i) {
+                if (units[i].u.y == units[i].u.z) continue;
+                int k = ucls[i] < 3 ? ucls[i] : -2;
+                // (a piece of a mixed box may still have one axis)
+                for (int r = units[i].u.y; k < 0 && k != -1 && r < units[i].u.z; ++r)
+                    for (int64_t j = ranges[r].x & kRangeIdx; j < ranges[r].y && k != -1; ++j) {
+                        const int kj = axis_of(j);
+                        k = (k == -2 || k == -3 - kj) && kj >= 0 ? -3 - kj : -1;
+                    }
+                if (k <= -3) k = -3 - k;
                 if (k >= 0) {
                     is_axis[i] = 1;
                     units[i].u.w |= k << 8;

@@ -64,6 +64,27 @@ __global__ void __launch_bounds__(256) k_slice(const double* __restrict__ v, int
     }
 }
 
+// 1/sqrt(x) for x in the normal range of floats: an FP32 estimate y (relative error below
+// 2^-21) and one step of Householder's third-order iteration, y (1 + e/2 + 3/8 e^2) with
+// e = 1 - x y^2, whose remainder 5/16 e^3 is below 2^-62.
+__device__ __forceinline__ double rsqrt3(double x) {
+    const double y = (double)rsqrtf((float)x);
+    const double e = fma(-(x * y), y, 1.0);
+    return fma(y * e, fma(0.375, e, 0.5), y);
+}
+
+// Nearest integer to x 2^(55 - e) (halves away from zero) for finite |x| < 2^e, from x's own
+// bits: the conversion would take the FP64 pipe.
+__device__ __forceinline__ long long fixed56(double x, int e) {
+    const long long u = __double_as_longlong(x);
+    const int ex = (int)((u >> 52) & 0x7ff);
+    if (ex == 0) return x == 0.0 ? 0LL : __double2ll_rn(scalbn(x, 55 - e));      // subnormal
+    const long long m = (u & 0xfffffffffffffLL) | 0x10000000000000LL;       // x = m 2^(ex - 1075)
+    const int sh = ex - 1075 + 55 - e;                                      // at most 2
+    long long y = sh >= 0 ? m << sh : (sh > -64 ? ((m >> (-sh - 1)) + 1) >> 1 : 0LL);
+    return u < 0 ? -y : y;
+}
+
 // One warp per target, NV kernel values a lane.
 template <int NV>
 __global__ void __launch_bounds__(128) k_slice_eval(const int* __restrict__ tleaf_of, int64_t t0, int n, int64_t nt,
@@ -82,25 +103,23 @@ __global__ void __launch_bounds__(128) k_slice_eval(const int* __restrict__ tlea
         x[d] = (txyz[d * nt + t] - ctr[3 * b + d]) / r;
         nv[d] = tnrm ? tnrm[d * nt + t] : (d == axis ? 1.0 : 0.0);
     }
-    double v[NV], m = 0.0;
-    bool fin = true;
+    double v[NV];
+    int top = 0;                                  // largest exponent field
 #pragma unroll
     for (int j = 0; j < NV; ++j) {
         const int k = j * 32 + lane;
         v[j] = 0.0;
         if (k < Q) {
             const double dx = x[0] - bpts[3 * k], dy = x[1] - bpts[3 * k + 1], dz = x[2] - bpts[3 * k + 2];
-            const double inv = rsqrt(dx * dx + dy * dy + dz * dz);
+            const double inv = rsqrt3(dx * dx + dy * dy + dz * dz);
             v[j] = grad ? (nv[0] * dx + nv[1] * dy + nv[2] * dz) * (inv * inv * inv) : inv;
         }
-        const double a = fabs(v[j]);
-        fin = fin && isfinite(a);
-        m = fmax(m, a);
+        top = max(top, (__double2hiint(v[j]) >> 20) & 0x7ff);
     }
 #pragma unroll
-    for (int o = 16; o; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-    fin = __all_sync(0xffffffffu, fin);
-    const int e = fin ? slice_exp(m) : 0;
+    for (int o = 16; o; o >>= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
+    const bool fin = top < 0x7ff;
+    const int e = fin ? top - 1022 : 0;           // |v| < 2^e
     if (lane == 0) {
         exps[i] = fin ? e : kNotFinite;
         oscale[i] = grad ? 1.0 / r : 1.0;
@@ -110,7 +129,7 @@ __global__ void __launch_bounds__(128) k_slice_eval(const int* __restrict__ tlea
     for (int j = 0; j < NV; ++j) {
         if (j * 32 >= Kc) break;
         __half d[kSlices];
-        slice_digits(fin ? __double2ll_rn(scale2(v[j], 55 - e)) : 0LL, d);
+        slice_digits(fin ? fixed56(v[j], e) : 0LL, d);
 #pragma unroll
         for (int s = 0; s < kSlices; ++s) o[(size_t)j * 32 * kSlices + s * 32] = d[s];
     }
