@@ -790,6 +790,11 @@ constexpr long long kRangeIdx = (1LL << 48) - 1;
 constexpr int kCloseBits = 5;
 __host__ __device__ inline int range_exp(long long fl) { return (int)((fl >> 48) & 255) - 128; }
 constexpr int kP2PUnitSrc = 2048;
+// A tree whose leaves give fewer than two waves of resident warps (two 8-warp blocks an
+// SM) takes smaller units, down to kP2PUnitMin sources: one warp walks its unit's sources
+// one chunk after the other, and a 16,000-point tree's 833 units of ~900 sources left most
+// of the chip idle for 150 us.
+constexpr int kP2PUnitMin = 128;
 // Larger target leaves of the single layer and the field go to the block kernel (a
 // thread per target, sources staged once per leaf).  The double layers always take the
 // warp kernel, in passes, for its exact products.
@@ -2294,6 +2299,28 @@ int setup(Plan& P, const double* src_nrm, const double* trg_nrm, cudaStream_t s)
         std::vector<signed char> ucls;         // DL: the dipole axis class of a unit's boxes
         auto half = [&](int box) { return std::ldexp(T.root_h, -T.h_lvl[box]); };
         auto exp_of = [](double ext) { return std::max(-100, std::min(100, std::ilogb(ext * (1.0 + 1e-12)) + 1)); };
+        // sources per unit: the most that still give two waves of units
+        int unit_src = kP2PUnitSrc;
+        {
+            const int kind = P.kernel == KIFMM_KERNEL_SL ? 0 : P.kernel == KIFMM_KERNEL_DL ? 1
+                                                             : P.kernel == KIFMM_KERNEL_ADL ? 2 : 3;
+            const int pt = 8 * (kind == 0 ? NearShape<0>::kMaxT : kind == 1 ? NearShape<1>::kMaxT
+                                : kind == 2 ? NearShape<2>::kMaxT : NearShape<3>::kMaxT);
+            std::vector<std::pair<int64_t, int64_t>> load(tleaf.size());   // (sources, passes) per leaf
+            for (size_t li = 0; li < tleaf.size(); ++li) {
+                int64_t src = 0;
+                for (int k = p2p_off[li]; k < p2p_off[li + 1]; ++k)
+                    src += T.h_rng[4 * p2p_idx[k] + 1] - T.h_rng[4 * p2p_idx[k]];
+                const int64_t ntg = T.h_rng[4 * tleaf[li] + 3] - T.h_rng[4 * tleaf[li] + 2];
+                load[li] = {src, (ntg + pt - 1) / pt};
+            }
+            const int64_t wanted = 2 * 2 * kP2PWarps * (int64_t)nsm;
+            for (; unit_src > kP2PUnitMin; unit_src /= 2) {
+                int64_t n = 0;
+                for (const auto& l : load) n += (l.first + unit_src - 1) / unit_src * l.second;
+                if (n >= wanted) break;
+            }
+        }
         // leaves are independent: blocks of them by thread, joined in leaf order
         constexpr size_t kLeafBlock = 128;
         const size_t nblk = (tleaf.size() + kLeafBlock - 1) / kLeafBlock;
@@ -2343,12 +2370,12 @@ int setup(Plan& P, const double* src_nrm, const double* trg_nrm, cudaStream_t s)
                     const long long ebits = (long long)(exp_of(box_ext) + 128) << 48;
                     int64_t j0 = T.h_rng[4 * a], j1 = T.h_rng[4 * a + 1];
                     while (j0 < j1) {
-                        const int64_t take = std::min<int64_t>(j1 - j0, kP2PUnitSrc - cnt);
+                        const int64_t take = std::min<int64_t>(j1 - j0, unit_src - cnt);
                         B.ranges.push_back(make_longlong2(j0 | ebits, j0 + take));
                         B.rleaf.push_back((int)li);
                         cnt += take;
                         j0 += take;
-                        if (cnt == kP2PUnitSrc) close_unit();
+                        if (cnt == unit_src) close_unit();
                     }
                 }
                 if (cnt > 0 || B.units.size() == u0) close_unit();

@@ -64,11 +64,12 @@ __global__ void __launch_bounds__(256) k_slice(const double* __restrict__ v, int
     }
 }
 
-// 1/sqrt(x) for x in the normal range of floats: an FP32 estimate y (relative error below
-// 2^-21) and one step of Householder's third-order iteration, y (1 + e/2 + 3/8 e^2) with
-// e = 1 - x y^2, whose remainder 5/16 e^3 is below 2^-62.
+// 1/sqrt(x) from the hardware's FP64 estimate y (its upper half: relative error below 2^-19)
+// and one step of Householder's third-order iteration, y (1 + e/2 + 3/8 e^2) with
+// e = 1 - x y^2, whose remainder 5/16 e^3 is below 2^-55.
 __device__ __forceinline__ double rsqrt3(double x) {
-    const double y = (double)rsqrtf((float)x);
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
     const double e = fma(-(x * y), y, 1.0);
     return fma(y * e, fma(0.375, e, 0.5), y);
 }
