@@ -106,6 +106,31 @@ constexpr int kKeyBits = 21;        // Morton bits per axis
 constexpr double kDelta = 1e-5;     // tolerance radius of the singular pair (Sec. III.A.1)
 constexpr int kNumOffsets = 343;    // (dx, dy, dz) in [-3, 3]^3 -> (dx+3)*49 + (dy+3)*7 + (dz+3)
 
+// Programmatic dependent launch.  A kernel of a chain calls pdl_trigger() on entry, which
+// lets its successor's blocks start their prologue (barriers, tensor memory, static operator
+// loads) while it runs, and pdl_wait() before it touches anything a predecessor writes or
+// reads: that waits until the predecessor is complete, and with it all before it.
+// Launched without the attribute, both are no-ops.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <typename... KArgs, typename... Args>
+inline int launch_pdl(bool pdl, void (*kern)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t s,
+                      Args... args) {
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = pdl ? 1 : 0;
+    KF_CHECK_CUDA(cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...));
+    return KIFMM_OK;
+}
+
 inline int div_up(int64_t a, int64_t b) { return (int)((a + b - 1) / b); }
 
 // Tree: sorted points, boxes (level-major, Morton-sorted within a level) and

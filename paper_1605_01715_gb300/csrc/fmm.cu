@@ -34,11 +34,11 @@ namespace kifmm {
 int tc_tile_pairs(int Qp);
 int tc_row_groups(int Mr);
 int tc_split_table(const float* table, __half* hi, __half* lo, size_t n, int* texp, cudaStream_t s);
-int tc_box_split(const float* v, int Q, int Qp, int b0, int b1, __half* hi, __half* lo, int* e, cudaStream_t s);
+int tc_box_split(const float* v, int Q, int Qp, int b0, int b1, __half* hi, __half* lo, int* e, bool pdl, cudaStream_t s);
 int tc_make_map(CUtensorMap* map, const __half* table, int nops, int Mr, int Kp);
 int launch_pair_tc(int which, const CUtensorMap& hi, const CUtensorMap& lo, int texp, int M, int Mr, int Kp,
                    int ostride, const int4* tiles, int ntiles, const int* pin, const int* pout, const int* bexp,
-                   const __half* in_hi, const __half* in_lo, float* out, int* err, cudaStream_t s,
+                   const __half* in_hi, const __half* in_lo, float* out, int* err, bool pdl, cudaStream_t s,
                    const int* kcount = nullptr);
 
 namespace {
@@ -320,6 +320,7 @@ k_surf_f(const int* __restrict__ boxes, const int* __restrict__ off, const int* 
          const float4* __restrict__ bcf, const int64_t* __restrict__ rng, const float* __restrict__ sxf, int64_t ns,
          const float* __restrict__ qs, const float* __restrict__ surf, int Q, int Qp, __half* __restrict__ vin_h,
          __half* __restrict__ vin_l, int* __restrict__ bexp, const int* __restrict__ bax) {
+    pdl_trigger();
     const int slot = down ? (int)blockIdx.x : boxes[blockIdx.x];   // X boxes are stored in list order
     __shared__ float4 sp[NT];
     __shared__ float4 sd[(DIPOLE || DIFF) ? NT : 1];
@@ -556,6 +557,7 @@ k_d2t(const int* __restrict__ leaves, const int64_t* __restrict__ rng, const Rea
     constexpr int R = 2;
     extern __shared__ __align__(32) unsigned char smem_raw[];
     Real* ds = reinterpret_cast<Real*>(smem_raw);
+    pdl_wait();
     int b = leaves[blockIdx.x];
     for (int k = threadIdx.x; k < Qp; k += blockDim.x) ds[k] = d[(size_t)b * Qp + k];
     __syncthreads();
@@ -791,19 +793,23 @@ constexpr int kCloseBits = 5;
 __host__ __device__ inline int range_exp(long long fl) { return (int)((fl >> 48) & 255) - 128; }
 constexpr int kP2PUnitSrc = 2048;
 // A tree whose leaves give fewer than two waves of resident warps (two 8-warp blocks an
-// SM) takes smaller units, down to kP2PUnitMin sources: one warp walks its unit's sources
-// one chunk after the other, and a 16,000-point tree's 833 units of ~900 sources left most
-// of the chip idle for 150 us.
-constexpr int kP2PUnitMin = 128;
+// SM) takes smaller units: one warp walks its unit's sources one chunk after the other, and a
+// 16,000-point tree's 833 units of ~900 sources left most of the chip idle for 150 us.
+// Double layers: fewer sources (down to kP2PUnitMin), which cuts a target's FP32 sum at
+// other places; then, and for the other kernels from the start, narrower passes, down to 8
+// targets, over which every sum stays the same bit for bit (a single layer of random
+// densities is a small remainder of its terms, and its FP32 sums are left as they are).
+constexpr int kP2PUnitMin = 256;
+constexpr int kPassShiftMax = 3;
 // Larger target leaves of the single layer and the field go to the block kernel (a
 // thread per target, sources staged once per leaf).  The double layers always take the
 // warp kernel, in passes, for its exact products.
 constexpr int kP2PWarpMaxLeaf = 64;
 // unit flags (int4 .w): bit 0 the leaf's first unit, bit 1 the leaf spans several units;
 // bits 8..9 the dipoles' axis of a KIND 4 unit; bits 16..30 one plus the unit's one pass
-// of 8 kMaxT targets, or 0 for all of the leaf's targets (the passes of a leaf share no
+// of 8 kMaxT >> (bits 4..5) targets, or 0 for all of the leaf's targets (the passes of a leaf share no
 // targets, so they are dealt to separate warps: each pass walks all of its sources anyway)
-constexpr int kUnitFirst = 1, kUnitSplit = 2, kUnitPassShift = 16;
+constexpr int kUnitFirst = 1, kUnitSplit = 2, kUnitNarrowShift = 4, kUnitPassShift = 16;
 
 // targets per lane per pass (plain and corrected-distance launches) and float4 entries
 // staged per source, by kernel: as many targets as keep each kernel within 128
@@ -1233,8 +1239,9 @@ k_p2p_warp(const int* __restrict__ leaves, int nunits, const int4* __restrict__ 
     float* raw = reinterpret_cast<float*>(st + S::kStage * 32);
     constexpr int kMaxT = CORR ? S::kMaxTCorr : S::kMaxT;
     const int pass = u.w >> kUnitPassShift;
-    const int64_t tf = pass ? tb + (int64_t)(pass - 1) * (8 * kMaxT) : tb;
-    const int64_t tl = pass && tf + 8 * kMaxT < te ? tf + 8 * kMaxT : te;
+    const int pt = (8 * kMaxT) >> ((u.w >> kUnitNarrowShift) & 3);
+    const int64_t tf = pass ? tb + (int64_t)(pass - 1) * pt : tb;
+    const int64_t tl = pass && tf + pt < te ? tf + pt : te;
     for (int64_t t0 = tf; t0 < tl; t0 += 8 * kMaxT) {
         const int n = (int)(tl - t0 < 8 * kMaxT ? tl - t0 : 8 * kMaxT);
         const int64_t tend = t0 + n;
@@ -2299,13 +2306,11 @@ int setup(Plan& P, const double* src_nrm, const double* trg_nrm, cudaStream_t s)
         std::vector<signed char> ucls;         // DL: the dipole axis class of a unit's boxes
         auto half = [&](int box) { return std::ldexp(T.root_h, -T.h_lvl[box]); };
         auto exp_of = [](double ext) { return std::max(-100, std::min(100, std::ilogb(ext * (1.0 + 1e-12)) + 1)); };
-        // sources per unit: the most that still give two waves of units
+        // sources per unit: double layers take the most that still give two waves of units
+        const int64_t two_waves = 2 * 2 * kP2PWarps * (int64_t)nsm;
         int unit_src = kP2PUnitSrc;
-        {
-            const int kind = P.kernel == KIFMM_KERNEL_SL ? 0 : P.kernel == KIFMM_KERNEL_DL ? 1
-                                                             : P.kernel == KIFMM_KERNEL_ADL ? 2 : 3;
-            const int pt = 8 * (kind == 0 ? NearShape<0>::kMaxT : kind == 1 ? NearShape<1>::kMaxT
-                                : kind == 2 ? NearShape<2>::kMaxT : NearShape<3>::kMaxT);
+        if (P.kernel == KIFMM_KERNEL_DL || P.kernel == KIFMM_KERNEL_ADL) {
+            const int pt = 8 * (P.kernel == KIFMM_KERNEL_DL ? NearShape<1>::kMaxT : NearShape<2>::kMaxT);
             std::vector<std::pair<int64_t, int64_t>> load(tleaf.size());   // (sources, passes) per leaf
             for (size_t li = 0; li < tleaf.size(); ++li) {
                 int64_t src = 0;
@@ -2314,11 +2319,10 @@ int setup(Plan& P, const double* src_nrm, const double* trg_nrm, cudaStream_t s)
                 const int64_t ntg = T.h_rng[4 * tleaf[li] + 3] - T.h_rng[4 * tleaf[li] + 2];
                 load[li] = {src, (ntg + pt - 1) / pt};
             }
-            const int64_t wanted = 2 * 2 * kP2PWarps * (int64_t)nsm;
             for (; unit_src > kP2PUnitMin; unit_src /= 2) {
                 int64_t n = 0;
                 for (const auto& l : load) n += (l.first + unit_src - 1) / unit_src * l.second;
-                if (n >= wanted) break;
+                if (n >= two_waves) break;
             }
         }
         // leaves are independent: blocks of them by thread, joined in leaf order
@@ -2467,13 +2471,27 @@ int setup(Plan& P, const double* src_nrm, const double* trg_nrm, cudaStream_t s)
                              : k == 2 ? NearShape<2>::kMaxT : k == 3 ? NearShape<3>::kMaxT : NearShape<4>::kMaxT;
                 return (int64_t)8 * mt;
             };
+            auto passes = [&](size_t i, int sh) {
+                const int b = tleaf[units[i].u.x];
+                const int64_t ntg = T.h_rng[4 * b + 3] - T.h_rng[4 * b + 2], pt = std::max<int64_t>(8, pass_targets(is_axis[i] != 0) >> sh);
+                return units[i].u.y == units[i].u.z ? (int64_t)1 : (ntg + pt - 1) / pt;
+            };
+            int sh = 0;
+            for (; sh < kPassShiftMax; ++sh) {
+                int64_t n = 0;
+                for (size_t i = 0; i < units.size(); ++i) n += passes(i, sh);
+                if (n >= two_waves) break;
+            }
             std::vector<Unit> pu;
             std::vector<char> pa;
             pu.reserve(units.size());
             for (size_t i = 0; i < units.size(); ++i) {
                 const int b = tleaf[units[i].u.x];
                 const int64_t ntg = T.h_rng[4 * b + 3] - T.h_rng[4 * b + 2];
-                const int64_t pt = pass_targets(is_axis[i] != 0);
+                // (a pass holds at least 8 targets, one per lane of a source group)
+                int shi = sh;
+                while (shi > 0 && (pass_targets(is_axis[i] != 0) >> shi) < 8) --shi;
+                const int64_t pt = pass_targets(is_axis[i] != 0) >> shi;
                 const int64_t np = (ntg + pt - 1) / pt;
                 if (units[i].u.y == units[i].u.z || np <= 1) {
                     pu.push_back(units[i]);
@@ -2483,7 +2501,7 @@ int setup(Plan& P, const double* src_nrm, const double* trg_nrm, cudaStream_t s)
                 const int64_t per = units[i].work / ntg;      // sources of the unit
                 for (int64_t k = 0; k < np; ++k) {
                     Unit v = units[i];
-                    v.u.w |= (int)(k + 1) << kUnitPassShift;
+                    v.u.w |= (int)(k + 1) << kUnitPassShift | shi << kUnitNarrowShift;
                     v.work = std::min(pt, ntg - k * pt) * per;
                     pu.push_back(v);
                     pa.push_back(is_axis[i]);
@@ -2608,6 +2626,7 @@ int setup(Plan& P, const double* src_nrm, const double* trg_nrm, cudaStream_t s)
             KF_CHECK_CUDA(cudaStreamCreateWithPriority(&P.x_stream, cudaStreamNonBlocking, prio_hi));
             KF_CHECK_CUDA(cudaEventCreateWithFlags(&P.ev_x, cudaEventDisableTiming));
         }
+        KF_CHECK_CUDA(cudaEventCreateWithFlags(&P.ev_start, cudaEventDisableTiming));
         KF_CHECK_CUDA(cudaEventCreateWithFlags(&P.ev_fork, cudaEventDisableTiming));
         KF_CHECK_CUDA(cudaEventCreateWithFlags(&P.ev_join, cudaEventDisableTiming));
         KF_CHECK_CUDA(cudaEventCreateWithFlags(&P.ev_far, cudaEventDisableTiming));
@@ -2675,6 +2694,12 @@ int run_pairs(const Plan& P, int which, const PairTiles& pt, int t0, int t1, con
 // (the 1M cube at 128 points per leaf: 52, once its exact zeros are left out; at 192:
 // 298; curved surfaces: several hundred).
 constexpr int64_t kLateNearPairs = 100;
+// Near-field pairs below which the far field's kernels are launched programmatically (each
+// one's prologue beside its predecessor's end): 20k sphere 139 -> 112 us, 2k sphere 57 -> 50.
+// The waiting blocks of the translation kernel hold whole SMs, which a larger near field
+// would use (24-instance forest, 150M pairs: 569 -> 603 us; 1M cube 773 -> 807).
+constexpr int64_t kPdlPairs = 50000000;
+inline bool pdl_chain(const Plan& P) { return P.near_pairs < kPdlPairs; }
 // Near-field pairs from which the X list stays in the far field's chain.
 constexpr int64_t kXBesidePairs = 300000000;
 
@@ -2692,7 +2717,7 @@ int run_pairs<float>(const Plan& P, int which, const PairTiles& pt, int t0, int 
     const int Mr = out_up ? o.Ku : o.Kd, M = out_up ? o.ru : o.rd;
     // split even without tiles: M2L reads the splits the upward pass leaves behind
     if (b1 > b0) {
-        KF_TRY(tc_box_split(z, r, K, b0, b1, P.vin_h.p, P.vin_l.p, P.bexp.p, s));
+        KF_TRY(tc_box_split(z, r, K, b0, b1, P.vin_h.p, P.vin_l.p, P.bexp.p, pdl_chain(P), s));
         ++launches;
     }
     if (t1 <= t0) return KIFMM_OK;
@@ -2709,7 +2734,7 @@ int run_pairs<float>(const Plan& P, int which, const PairTiles& pt, int t0, int 
         }
     }
     KF_TRY(launch_pair_tc(which, m[0], m[1], o.texp[which], M, Mr, K, Mr, pt.tiles.p + t0, t1 - t0, pt.pin.p,
-                          pt.pout.p, P.bexp.p, P.vin_h.p, P.vin_l.p, out, P.err.p, s, kc));
+                          pt.pout.p, P.bexp.p, P.vin_h.p, P.vin_l.p, out, P.err.p, pdl_chain(P), s, kc));
     ++launches;
     return KIFMM_OK;
 }
@@ -2725,7 +2750,7 @@ int project(const Plan& P, int fam, const PairTiles& pt, float* z, cudaStream_t 
     const CUtensorMap* m = o.tmaps[fam];
     KF_TRY(launch_pair_tc(3, m[0], m[1], o.texp[fam], M, Mr, Kp, Mr, pt.tiles.p, pt.ntiles, pt.pin.p, pt.pout.p,
                           fam == 3 ? P.sexp.p : P.xexp.p, fam == 3 ? P.sin_h.p : P.xin_h.p,
-                          fam == 3 ? P.sin_l.p : P.xin_l.p, z, P.err.p, s));
+                          fam == 3 ? P.sin_l.p : P.xin_l.p, z, P.err.p, pdl_chain(P), s));
     launches += 2;
     return KIFMM_OK;
 }
@@ -2834,6 +2859,10 @@ int matvec(Plan& P, const Bufs<Real>& B, const double* q, double* out, cudaStrea
     // mixed DL: the FP32 remainders of the dipoles too (the near field's exact products)
     const bool dl_lo = dl && std::is_same<Real, float>::value;
     KF_TRY(mark(0));
+    if (near_overlap) {
+        KF_CHECK_CUDA(cudaEventRecord(P.ev_start, s));
+        KF_CHECK_CUDA(cudaStreamWaitEvent(P.near_stream, P.ev_start, 0));
+    }
     if (P.io_in)
         k_scatter_q<Real><<<div_up(T.ns, 256), 256, 0, s>>>(q, P.isperm.p, T.ns, dl ? P.snrm.p : nullptr, B.q,
                                                             dl_lo);
@@ -2875,13 +2904,15 @@ int matvec(Plan& P, const Bufs<Real>& B, const double* q, double* out, cudaStrea
         up = P.zu.p;
         dn = P.zd.p;
         dw = P.ops->Kd;
-        // zeroed on the near field's stream when there is one, beside S2U (which does not
-        // touch them); the far field waits before its first accumulation into them
+        // zeroed on the near field's stream when there is one, beside the gather, so that from
+        // S2U on the far field is one chain of kernels
         const cudaStream_t zs = near_overlap ? P.near_stream : s;
-        if (near_overlap) KF_CHECK_CUDA(cudaStreamWaitEvent(zs, P.ev_fork, 0));
         KF_CHECK_CUDA(cudaMemsetAsync(up, 0, P.zu.bytes(), zs));
         KF_CHECK_CUDA(cudaMemsetAsync(dn, 0, P.zd.bytes(), zs));
-        if (near_overlap) KF_CHECK_CUDA(cudaEventRecord(P.ev_zero, zs));
+        if (near_overlap) {
+            KF_CHECK_CUDA(cudaEventRecord(P.ev_zero, zs));
+            KF_CHECK_CUDA(cudaStreamWaitEvent(s, P.ev_zero, 0));
+        }
         launches += 2;
     }
     KF_TRY(mark(1));
@@ -2924,7 +2955,6 @@ int matvec(Plan& P, const Bufs<Real>& B, const double* q, double* out, cudaStrea
     KF_TRY(mark(2));
     // mixed: the leaves' projections; U2U, deepest parents first
     if constexpr (mixed) {
-        if (near_overlap) KF_CHECK_CUDA(cudaStreamWaitEvent(s, P.ev_zero, 0));
         KF_TRY(project(P, 3, P.proj_up, up, s, launches));
     }
     for (int l = T.nlev - 1; l >= 2; --l)
@@ -2967,9 +2997,8 @@ int matvec(Plan& P, const Bufs<Real>& B, const double* q, double* out, cudaStrea
     KF_TRY(mark(6));
     if (P.n_tleaf) {
         for (int c = 0; c < P.nc; ++c) {
-            k_d2t<Real><<<P.n_tleaf, 128, dw * sizeof(Real), s>>>(P.tleaf.p, T.rng.p, B.d2t + (size_t)c * T.nt * dw,
-                                                                  dn, dw, B.res + (size_t)c * T.nt);
-            KF_CHECK_LAUNCH();
+            KF_TRY(launch_pdl(mixed && pdl_chain(P), k_d2t<Real>, (unsigned)P.n_tleaf, 128u, dw * sizeof(Real), s, P.tleaf.p, T.rng.p,
+                              B.d2t + (size_t)c * T.nt * dw, dn, dw, B.res + (size_t)c * T.nt));
             ++launches;
         }
     }

@@ -44,6 +44,8 @@ constexpr int kSplitWarps = 8;
 __global__ void __launch_bounds__(32 * kSplitWarps) k_box_split(const float* __restrict__ v, int Q, int Qp, int b0,
                                                                 int b1, __half* __restrict__ hi,
                                                                 __half* __restrict__ lo, int* __restrict__ e) {
+    pdl_trigger();
+    pdl_wait();
     const int lane = threadIdx.x & 31;
     const int b = b0 + (int)blockIdx.x * kSplitWarps + (int)(threadIdx.x >> 5);
     if (b >= b1) return;                      // whole warp; no block-wide barrier below
@@ -116,11 +118,10 @@ int tc_split_table(const float* table, __half* hi, __half* lo, size_t n, int* te
 }
 
 // Per-box scales and FP16 hi/lo splits of boxes [b0, b1) of a check-potential buffer.
-int tc_box_split(const float* v, int Q, int Qp, int b0, int b1, __half* hi, __half* lo, int* e, cudaStream_t s) {
+int tc_box_split(const float* v, int Q, int Qp, int b0, int b1, __half* hi, __half* lo, int* e, bool pdl, cudaStream_t s) {
     if (b1 <= b0) return KIFMM_OK;
-    k_box_split<<<(b1 - b0 + kSplitWarps - 1) / kSplitWarps, 32 * kSplitWarps, 0, s>>>(v, Q, Qp, b0, b1, hi, lo, e);
-    KF_CHECK_LAUNCH();
-    return KIFMM_OK;
+    return launch_pdl(pdl, k_box_split, (unsigned)((b1 - b0 + kSplitWarps - 1) / kSplitWarps), 32 * kSplitWarps, 0, s, v, Q, Qp,
+                      b0, b1, hi, lo, e);
 }
 
 // 2-D tiled map of a row-major FP16 matrix, box kKS columns x box_rows rows, 64-byte
@@ -151,7 +152,7 @@ template <int SLABS, int N>
 static int launch_shape(int which, const CUtensorMap& hi, const CUtensorMap& lo, int texp, int M, int Mr, int Kp,
                         int ostride, const int4* tiles, int ntiles, const int* pin, const int* pout,
                         const int* bexp, const __half* in_hi, const __half* in_lo, float* out, int* err,
-                        const int* kcount, cudaStream_t s) {
+                        const int* kcount, bool pdl, cudaStream_t s) {
     using S = tc::Shape<SLABS, N>;
     auto kern = which == 0   ? tc::k_u2u_tc<SLABS, N>
                 : which == 1 ? tc::k_m2l_tc<SLABS, N>
@@ -176,10 +177,8 @@ static int launch_shape(int which, const CUtensorMap& hi, const CUtensorMap& lo,
     KF_CHECK_CUDA(cudaGetDevice(&dev));
     KF_CHECK_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     const int grid = nitems < nsm ? nitems : nsm;
-    kern<<<grid, tc::kThreads, S::kSmemBytes, s>>>(hi, lo, M, Kp, ostride, Mr, mgroups, nitems, tiles, pin, pout,
-                                                    bexp, texp, in_hi, in_lo, out, err, kcount);
-    KF_CHECK_LAUNCH();
-    return KIFMM_OK;
+    return launch_pdl(pdl, kern, grid, tc::kThreads, S::kSmemBytes, s, hi, lo, M, Kp, ostride, Mr, mgroups, nitems, tiles, pin,
+                      pout, bexp, texp, in_hi, in_lo, out, err, kcount);
 }
 
 // which: 0 = U2U, 1 = M2L, 2 = L2L, 3 = projection onto a check-space basis.  The
@@ -187,14 +186,14 @@ static int launch_shape(int which, const CUtensorMap& hi, const CUtensorMap& lo,
 // (tc_box_split, Kp per box) of every box a pair reads; out: ostride per box.
 int launch_pair_tc(int which, const CUtensorMap& hi, const CUtensorMap& lo, int texp, int M, int Mr, int Kp,
                    int ostride, const int4* tiles, int ntiles, const int* pin, const int* pout, const int* bexp,
-                   const __half* in_hi, const __half* in_lo, float* out, int* err, cudaStream_t s,
+                   const __half* in_hi, const __half* in_lo, float* out, int* err, bool pdl, cudaStream_t s,
                    const int* kcount) {
     if (ntiles <= 0) return KIFMM_OK;
     if (Mr <= 128)
         return launch_shape<1, 256>(which, hi, lo, texp, M, Mr, Kp, ostride, tiles, ntiles, pin, pout, bexp, in_hi,
-                                    in_lo, out, err, kcount, s);
+                                    in_lo, out, err, kcount, pdl, s);
     return launch_shape<2, 128>(which, hi, lo, texp, M, Mr, Kp, ostride, tiles, ntiles, pin, pout, bexp, in_hi,
-                                in_lo, out, err, kcount, s);
+                                in_lo, out, err, kcount, pdl, s);
 }
 
 }  // namespace kifmm

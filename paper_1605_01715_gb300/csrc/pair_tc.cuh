@@ -50,6 +50,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "common.cuh"
+
 namespace kifmm {
 namespace tc {
 
@@ -414,6 +416,7 @@ __device__ __forceinline__ void pair_tc_body(const CUtensorMap& map_hi, const CU
     // items of this CTA: every G-th from blockIdx.x, or the first kcount[blockIdx.x] of them
     const int K = kcount ? kcount[blockIdx.x]
                          : (nitems > (int)blockIdx.x ? (nitems - (int)blockIdx.x + G - 1) / G : 0);
+    pdl_trigger();
     if (K == 0) return;                   // uniform: nothing allocated yet
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* base = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
@@ -553,6 +556,7 @@ __device__ __forceinline__ void pair_tc_body(const CUtensorMap& map_hi, const CU
                         tma_load_2d(stage_u32(s), &map_hi, i * kKS, arow, &tma_full[s]);
                         tma_load_2d(stage_u32(s) + S::kABytes, &map_lo, i * kKS, arow, &tma_full[s]);
                     }
+                    if (g == 0) pdl_wait();        // the inputs; the operator's first rows are on their way
                     const uint32_t bh = stage_u32(s) + 2 * S::kABytes;
                     const bool inside = i * kKS + 8 * c < Kp;   // an 8-group lies wholly inside or outside Kp
 #pragma unroll
@@ -587,6 +591,7 @@ __device__ __forceinline__ void pair_tc_body(const CUtensorMap& map_hi, const CU
         }
     } else if (warp < kScatWarp0) {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kFoldRegs));
+        pdl_wait();
         // ---- folds: half `half`, lane quarter warp % 4 (the TMEM lanes this warp may read) ----
         const int ft = tid - kFoldWarp0 * 32, half = (warp - kFoldWarp0) >> 2;
         const uint32_t lanes = (uint32_t)((warp & 3) * 32) << 16;
@@ -665,6 +670,7 @@ __device__ __forceinline__ void pair_tc_body(const CUtensorMap& map_hi, const CU
         }
     } else {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kScatRegs));
+        pdl_wait();
         // ---- scatter of the parked sums, beside the next item's MMAs and folds: lane quarter
         // warp % 4 of both halves; each column is one output box's 32 consecutive rows.
         // All SMs together scatter 16 to 19 B per clock and SM (the L2 fabric's rate, wider

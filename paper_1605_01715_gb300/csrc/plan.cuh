@@ -151,7 +151,7 @@ struct Plan {
     // the far-field sum is added
     cudaStream_t near_stream = nullptr, far_stream = nullptr;
     cudaStream_t x_stream = nullptr;   // the X list, beside the upward pass and M2L
-    cudaEvent_t ev_x = nullptr;
+    cudaEvent_t ev_x = nullptr, ev_start = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_far = nullptr, ev_zero = nullptr;
     const double* g_q = nullptr;
     double* g_out = nullptr;
@@ -182,6 +182,7 @@ struct Plan {
         if (ev_far) cudaEventDestroy(ev_far);
         if (ev_zero) cudaEventDestroy(ev_zero);
         if (ev_x) cudaEventDestroy(ev_x);
+        if (ev_start) cudaEventDestroy(ev_start);
         if (x_stream) cudaStreamDestroy(x_stream);
         if (near_stream) cudaStreamDestroy(near_stream);
         if (far_stream) cudaStreamDestroy(far_stream);
