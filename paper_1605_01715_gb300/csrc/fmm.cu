@@ -70,8 +70,27 @@ template <> struct RT<double> {
 inline bool gradient_kernel(int kernel) { return kernel == KIFMM_KERNEL_ADL || kernel == KIFMM_KERNEL_FIELD; }
 
 // ---------------------------------------------------------------- gather
-// lo: also write the rounding remainders of the dipoles (3 more rows, read by the
-// mixed near field's exact products)
+// Dipole v n_i of sorted position i, SoA; lo: also the rounding remainders (3 more rows,
+// read by the mixed near field's exact products).  Products and conversions take the FP64
+// pipe, 15 operations a point at 2 a clock, which bound the gather; a zero component of
+// the normal (flat faces normal to an axis) needs none.
+template <typename Real>
+__device__ __forceinline__ void store_dipole(double v, const double* __restrict__ snrm, int64_t n, int64_t i,
+                                             Real* __restrict__ qs, bool lo) {
+    const bool finite = (__double2hiint(v) & 0x7ff00000) != 0x7ff00000;
+    for (int d = 0; d < 3; ++d) {
+        const double nd = snrm[d * n + i];
+        Real hi = 0, rest = 0;
+        if (!finite || (__double2hiint(nd) << 1 | __double2loint(nd)) != 0) {
+            const double pd = v * nd;
+            hi = (Real)pd;
+            if (lo) rest = (Real)(pd - (double)hi);
+        }
+        qs[d * n + i] = hi;
+        if (lo) qs[(3 + d) * n + i] = rest;
+    }
+}
+
 template <typename Real>
 __global__ void k_gather_q(const double* __restrict__ q, const int64_t* __restrict__ perm, int64_t n,
                            const double* __restrict__ snrm, Real* __restrict__ qs, bool lo) {
@@ -79,11 +98,7 @@ __global__ void k_gather_q(const double* __restrict__ q, const int64_t* __restri
     if (i >= n) return;
     double v = q[perm[i]];
     if (snrm) {  // dipole strengths q n_j, SoA
-        for (int d = 0; d < 3; ++d) {
-            const double pd = v * snrm[d * n + i];
-            qs[d * n + i] = (Real)pd;
-            if (lo) qs[(3 + d) * n + i] = (Real)(pd - (double)(Real)pd);
-        }
+        store_dipole(v, snrm, n, i, qs, lo);
     } else {
         qs[i] = (Real)v;
     }
@@ -99,11 +114,7 @@ __global__ void k_scatter_q(const double* __restrict__ q, const int64_t* __restr
     const double v = q[i];
     const int64_t j = iperm[i];
     if (snrm) {
-        for (int d = 0; d < 3; ++d) {
-            const double pd = v * snrm[d * n + j];
-            qs[d * n + j] = (Real)pd;
-            if (lo) qs[(3 + d) * n + j] = (Real)(pd - (double)(Real)pd);
-        }
+        store_dipole(v, snrm, n, j, qs, lo);
     } else {
         qs[j] = (Real)v;
     }
@@ -793,13 +804,11 @@ constexpr int kCloseBits = 5;
 __host__ __device__ inline int range_exp(long long fl) { return (int)((fl >> 48) & 255) - 128; }
 constexpr int kP2PUnitSrc = 2048;
 // A tree whose leaves give fewer than two waves of resident warps (two 8-warp blocks an
-// SM) takes smaller units: one warp walks its unit's sources one chunk after the other, and a
-// 16,000-point tree's 833 units of ~900 sources left most of the chip idle for 150 us.
-// Double layers: fewer sources (down to kP2PUnitMin), which cuts a target's FP32 sum at
-// other places; then, and for the other kernels from the start, narrower passes, down to 8
-// targets, over which every sum stays the same bit for bit (a single layer of random
-// densities is a small remainder of its terms, and its FP32 sums are left as they are).
-constexpr int kP2PUnitMin = 256;
+// SM) takes narrower passes, down to 8 targets: one warp walks its unit's sources one chunk
+// after the other, and few units leave most of the chip idle behind the longest (near field
+// alone: 20k-point sphere 100 -> 72 us, 16,000-point pack 149 -> 113).  Every target's sum
+// stays the same bit for bit.  (Smaller units of sources reach 32 and 67 us, but cut a
+// target's FP32 sum at other places.)
 constexpr int kPassShiftMax = 3;
 // Larger target leaves of the single layer and the field go to the block kernel (a
 // thread per target, sources staged once per leaf).  The double layers always take the
@@ -813,10 +822,13 @@ constexpr int kUnitFirst = 1, kUnitSplit = 2, kUnitNarrowShift = 4, kUnitPassShi
 
 // targets per lane per pass (plain and corrected-distance launches) and float4 entries
 // staged per source, by kernel: as many targets as keep each kernel within 128
-// registers, so two blocks share an SM
+// registers, so two blocks share an SM (the double layer's 6 spill a little and still win:
+// staging a chunk of sources costs a pass about half of what its pairs do, and a leaf of 48
+// targets is one pass.  1M sphere, near field alone: 4 targets 1611 us, 5 1694, 6 1532, 8
+// 1549; the adjoint's 6 lose, 64-sphere pack 1027 -> 1063)
 template <int KIND> struct NearShape;
 template <> struct NearShape<0> { static constexpr int kMaxT = 8, kMaxTCorr = 6, kStage = 4, kRaw = 7; };
-template <> struct NearShape<1> { static constexpr int kMaxT = 4, kMaxTCorr = 4, kStage = 7, kRaw = 12; };
+template <> struct NearShape<1> { static constexpr int kMaxT = 6, kMaxTCorr = 4, kStage = 7, kRaw = 12; };
 template <> struct NearShape<2> { static constexpr int kMaxT = 4, kMaxTCorr = 2, kStage = 7, kRaw = 7; };
 template <> struct NearShape<3> { static constexpr int kMaxT = 8, kMaxTCorr = 6, kStage = 4, kRaw = 7; };
 // 4: the double layer on a unit whose dipoles all lie along one coordinate axis (flat
@@ -868,6 +880,19 @@ __device__ __forceinline__ void offset_forms(float a, float rest, float magic, f
     }
 }
 
+// a + b (packed, round to nearest), not moved out of the loop it stands in
+__device__ __forceinline__ float2 add2_here(float2 a, float2 b) {
+    float2 d;
+    asm volatile(
+        "{\n\t.reg .b64 x, y, z;\n\t"
+        "mov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\t"
+        "add.rn.f32x2 z, x, y;\n\t"
+        "mov.b64 {%0, %1}, z;\n\t}"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
+
 template <int KIND, int T, bool CORR>
 __device__ __forceinline__ void p2p_pass(int lane, int e0, int e1, const longlong2* __restrict__ ranges, int flags,
                                          float4 cb0, float4 cb1, const float* __restrict__ sxf, int64_t ns,
@@ -888,7 +913,11 @@ __device__ __forceinline__ void p2p_pass(int lane, int e0, int e1, const longlon
     // targets: offsets from the leaf centre, formed from FP32 hi/lo coordinates exactly as
     // the sources' below (a target and the same point as a source agree bit for bit), and
     // for the double layers split on the grid of the current range's exponent
-    float2 tfx[TP], tfy[TP], tfz[TP], acc[TP], acc2[NC > 1 ? TP : 1], acc3[NC > 1 ? TP : 1];
+    // FLY (the double layer's wide passes): the full offset is hi + lo, formed anew for each
+    // source instead of held: two thirds of the registers per target
+    constexpr bool FLY = KIND == 1 && !CORR && T > 4;
+    constexpr int TF = FLY ? 1 : TP;
+    float2 tfx[TF], tfy[TF], tfz[TF], acc[TP], acc2[NC > 1 ? TP : 1], acc3[NC > 1 ? TP : 1];
     float2 thx[ACC ? TP : 1], thy[ACC ? TP : 1], thz[ACC ? TP : 1];   // DL: t hi;  ADL: n hi
     float2 tlx[ACC ? TP : 1], tly[ACC ? TP : 1], tlz[ACC ? TP : 1];   // DL: t lo;  ADL: -n lo
     float2 tca[KIND == 2 ? TP : 1], tcb[KIND == 2 ? TP : 1];          // ADL: -n_hi.t_hi, -(n_hi.t_lo + n_lo.t)
@@ -935,9 +964,11 @@ __device__ __forceinline__ void p2p_pass(int lane, int e0, int e1, const longlon
                                __fmaf_rn(nh[2], tl[2], __fmaf_rn(nh[1], tl[1], __fmul_rn(nh[0], tl[0]))))));
                 }
             }
-            tfx[m] = make_float2(c[0][0], c[1][0]);
-            tfy[m] = make_float2(c[0][1], c[1][1]);
-            tfz[m] = make_float2(c[0][2], c[1][2]);
+            if (!FLY) {
+                tfx[m] = make_float2(c[0][0], c[1][0]);
+                tfy[m] = make_float2(c[0][1], c[1][1]);
+                tfz[m] = make_float2(c[0][2], c[1][2]);
+            }
             if (ACC) {
                 thx[m] = make_float2(c[0][3], c[1][3]);
                 thy[m] = make_float2(c[0][4], c[1][4]);
@@ -1098,7 +1129,8 @@ __device__ __forceinline__ void p2p_pass(int lane, int e0, int e1, const longlon
                 }
             }
             __syncwarp();
-            constexpr int kJJ = (KIND == 1 && CORR) ? 1 : 2;   // two sources in flight; the DL corrected launch would spill
+            // two sources in flight; the double layer's wide passes and its corrected launch hold no more
+            constexpr int kJJ = KIND == 1 && (CORR || T > 4) ? 1 : 2;
     #pragma unroll kJJ
             for (int jj = g; jj < cnt; jj += 4) {
                 const float4 A = st[jj], B = st[32 + jj];
@@ -1127,8 +1159,10 @@ __device__ __forceinline__ void p2p_pass(int lane, int e0, int e1, const longlon
                 }
     #pragma unroll
                 for (int m = 0; m < TP; ++m) {
-                    float2 dx = __fadd2_rn(tfx[m], lo2(A)), dy = __fadd2_rn(tfy[m], hi2(A)),
-                           dz = __fadd2_rn(tfz[m], lo2(B));
+                    const float2 fx = FLY ? add2_here(thx[m], tlx[m]) : tfx[m];
+                    const float2 fy = FLY ? add2_here(thy[m], tly[m]) : tfy[m];
+                    const float2 fz = FLY ? add2_here(thz[m], tlz[m]) : tfz[m];
+                    float2 dx = __fadd2_rn(fx, lo2(A)), dy = __fadd2_rn(fy, hi2(A)), dz = __fadd2_rn(fz, lo2(B));
                     if (CORR) {
                         // t - s = (tf - sf) + (te - se): the first difference is exact for close
                         // points, the second carries what FP32 offsets dropped
@@ -1161,7 +1195,7 @@ __device__ __forceinline__ void p2p_pass(int lane, int e0, int e1, const longlon
                         // m_hi . t_hi - a_j (exact) + m_hi . t_lo + m_lo . t - b_j
                         const float2 nh = __ffma2_rn(lo2(D), thz[m], __ffma2_rn(hi2(C), thy[m],
                                           __ffma2_rn(lo2(C), thx[m], hi2(B))));
-                        const float2 cr = __ffma2_rn(lo2(G), tfz[m], __ffma2_rn(hi2(F), tfy[m], __ffma2_rn(lo2(F), tfx[m],
+                        const float2 cr = __ffma2_rn(lo2(G), fz, __ffma2_rn(hi2(F), fy, __ffma2_rn(lo2(F), fx,
                                           __ffma2_rn(lo2(D), tlz[m], __ffma2_rn(hi2(C), tly[m],
                                           __ffma2_rn(lo2(C), tlx[m], hi2(D)))))));
                         num = __fadd2_rn(nh, cr);
@@ -2306,25 +2340,7 @@ int setup(Plan& P, const double* src_nrm, const double* trg_nrm, cudaStream_t s)
         std::vector<signed char> ucls;         // DL: the dipole axis class of a unit's boxes
         auto half = [&](int box) { return std::ldexp(T.root_h, -T.h_lvl[box]); };
         auto exp_of = [](double ext) { return std::max(-100, std::min(100, std::ilogb(ext * (1.0 + 1e-12)) + 1)); };
-        // sources per unit: double layers take the most that still give two waves of units
         const int64_t two_waves = 2 * 2 * kP2PWarps * (int64_t)nsm;
-        int unit_src = kP2PUnitSrc;
-        if (P.kernel == KIFMM_KERNEL_DL || P.kernel == KIFMM_KERNEL_ADL) {
-            const int pt = 8 * (P.kernel == KIFMM_KERNEL_DL ? NearShape<1>::kMaxT : NearShape<2>::kMaxT);
-            std::vector<std::pair<int64_t, int64_t>> load(tleaf.size());   // (sources, passes) per leaf
-            for (size_t li = 0; li < tleaf.size(); ++li) {
-                int64_t src = 0;
-                for (int k = p2p_off[li]; k < p2p_off[li + 1]; ++k)
-                    src += T.h_rng[4 * p2p_idx[k] + 1] - T.h_rng[4 * p2p_idx[k]];
-                const int64_t ntg = T.h_rng[4 * tleaf[li] + 3] - T.h_rng[4 * tleaf[li] + 2];
-                load[li] = {src, (ntg + pt - 1) / pt};
-            }
-            for (; unit_src > kP2PUnitMin; unit_src /= 2) {
-                int64_t n = 0;
-                for (const auto& l : load) n += (l.first + unit_src - 1) / unit_src * l.second;
-                if (n >= two_waves) break;
-            }
-        }
         // leaves are independent: blocks of them by thread, joined in leaf order
         constexpr size_t kLeafBlock = 128;
         const size_t nblk = (tleaf.size() + kLeafBlock - 1) / kLeafBlock;
@@ -2374,12 +2390,12 @@ int setup(Plan& P, const double* src_nrm, const double* trg_nrm, cudaStream_t s)
                     const long long ebits = (long long)(exp_of(box_ext) + 128) << 48;
                     int64_t j0 = T.h_rng[4 * a], j1 = T.h_rng[4 * a + 1];
                     while (j0 < j1) {
-                        const int64_t take = std::min<int64_t>(j1 - j0, unit_src - cnt);
+                        const int64_t take = std::min<int64_t>(j1 - j0, kP2PUnitSrc - cnt);
                         B.ranges.push_back(make_longlong2(j0 | ebits, j0 + take));
                         B.rleaf.push_back((int)li);
                         cnt += take;
                         j0 += take;
-                        if (cnt == unit_src) close_unit();
+                        if (cnt == kP2PUnitSrc) close_unit();
                     }
                 }
                 if (cnt > 0 || B.units.size() == u0) close_unit();
