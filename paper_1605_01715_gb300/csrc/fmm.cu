@@ -691,7 +691,10 @@ __global__ void k_p2p(const int* __restrict__ order, const int* __restrict__ lea
         };
         auto term = [&](const R4& y, const R2* yd, Real& dx, Real& dy, Real& dz, Real& w, Real& v) {
             dx = xt - y.x, dy = yt - y.y, dz = zt - y.z;
-            const Real r2 = dx * dx + dy * dy + dz * dz;
+            // (the single layer's order of the fused sum is written out: its terms nearly cancel
+            // for random densities, and another order moves the result by twice what two runs
+            // differ by)
+            const Real r2 = KIND == 0 ? fma(dz, dz, fma(dx, dx, dy * dy)) : dx * dx + dy * dy + dz * dz;
             const Real inv = RT<Real>::rsq(r2);
             w = v = 0;
             if (KIND == 3) {
