@@ -180,6 +180,13 @@ __device__ __forceinline__ bool mbar_wait_ab(uint64_t* bar, uint32_t parity, vol
     return false;
 }
 
+// The same for a whole warp that goes on to warp-wide (.aligned) instructions: lanes watch
+// the barrier and *abort on their own, so a barrier that completes as the flag is raised
+// can let some pass and others give up.  Every lane returns whether all of them passed.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort) {
+    return __all_sync(0xffffffffu, mbar_wait_ab(bar, parity, abort));
+}
+
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
@@ -630,7 +637,7 @@ __device__ __forceinline__ void pair_tc_body(const CUtensorMap& map_hi, const CU
             float msc = 1.f;
             bool ok = true;
             for (int j = 0; j < nst; ++j) {
-                if (!mbar_wait_ab(&acc_full[half], (uint32_t)((k * nst + j) & 1), abort)) {
+                if (!mbar_wait_warp(&acc_full[half], (uint32_t)((k * nst + j) & 1), abort)) {
                     ok = false;
                     break;
                 }
@@ -647,9 +654,9 @@ __device__ __forceinline__ void pair_tc_body(const CUtensorMap& map_hi, const CU
             if (ft < N) s_oscale[mbn][ft] = msc;
             // hand the sums to the scatter warps, once those have read the item before's
             if (ok && !cont) {
-                if (parked > 0) ok = mbar_wait_ab(&park_empty, (uint32_t)((parked - 1) & 1), abort);
+                if (parked > 0) ok = mbar_wait_warp(&park_empty, (uint32_t)((parked - 1) & 1), abort);
                 tc_fence_after();
-                if (__all_sync(0xffffffffu, ok)) {
+                if (ok) {
                     const uint32_t pk = tmem + lanes + (uint32_t)(S::kPark + half * 128);
 #pragma unroll
                     for (int j = 0; j < 128; j += 32) {

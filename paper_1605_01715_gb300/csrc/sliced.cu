@@ -328,7 +328,7 @@ k_sliced(const __grid_constant__ CUtensorMap map, int64_t plane_rows, const int*
             for (int j = 0; j < 32; ++j) sum[j] = 0.0;
             bool ok = true;
             for (int i0 = 0; i0 < nst; i0 += kOzChunk, ++f) {
-                if (!mbar_wait_ab(&acc_full, (uint32_t)(f & 1), abort)) {
+                if (!mbar_wait_warp(&acc_full, (uint32_t)(f & 1), abort)) {
                     ok = false;
                     break;
                 }
@@ -347,7 +347,7 @@ k_sliced(const __grid_constant__ CUtensorMap map, int64_t plane_rows, const int*
                     for (int c = 0; c < 8; ++c) sum[c0 + c] += join_digits(v, c);
                 }
             }
-            if (!__all_sync(0xffffffffu, ok)) break;
+            if (!ok) break;
             if (row < (STORE ? ostride : M)) {
 #pragma unroll
                 for (int j = 0; j < 32; ++j) {
