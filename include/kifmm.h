@@ -336,6 +336,7 @@ int kifmm_plan_profile(kifmm_plan plan, int enable, double* phases);
  * tensor-core translation GEMMs bound every pipeline wait; a wait that gives up
  * records a code in a device word of the plan, skips its writes and frees its
  * tensor memory.  Returns KIFMM_ERR_TIMEOUT if that ever happened, else KIFMM_OK.
+ * (kifmm_fmm_setup makes this check of its own kernels and fails with that status.)
  */
 int kifmm_plan_check(kifmm_plan plan);
 

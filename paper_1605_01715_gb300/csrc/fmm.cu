@@ -1884,6 +1884,19 @@ int build_projected(Plan& P, const HostPinv& h, OpTables* t, const std::vector<d
     return KIFMM_OK;
 }
 
+// KIFMM_ERR_TIMEOUT if a bounded wait of a kernel given the error word err has given up by
+// the end of the work on s, which is waited for.
+int check_waits(const int* err, cudaStream_t s) {
+    int h = 0;
+    KF_CHECK_CUDA(cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, s));
+    KF_CHECK_CUDA(cudaStreamSynchronize(s));
+    if (h) {
+        set_error("a tensor-core kernel gave up waiting on its pipeline (code %d)", h);
+        return KIFMM_ERR_TIMEOUT;
+    }
+    return KIFMM_OK;
+}
+
 // Per-target evaluation rows of the mixed form, G(x_t, 2.95 s) W_d (rd wide, stored Kd):
 // an FP64 product (W_d carries factors 1 / sigma, and its terms cancel to O(1)), rounded
 // once to FP32.  The kernel values of a chunk of targets are written as exact slices and
@@ -1933,8 +1946,8 @@ int build_d2t_sliced(Plan& P, const HostPinv& h, const std::vector<int>& tleaf_o
                                               div_up(n, kSlicePairs), dio.p, dio.p, sl.p, dexp.p, dos.p,
                                               out + ((size_t)c * nt + t0) * Kd, Kd, P.err.p, s));
         }
-    KF_CHECK_CUDA(cudaStreamSynchronize(s));   // the scratch is freed on return
-    return KIFMM_OK;
+    // (a copy to the host synchronizes: the scratch is freed on return)
+    return check_waits(P.err.p, s);
 }
 
 // The same of the FP64 form, G(x_t, 2.95 s) Pd (Q wide, stored Qp).
@@ -3374,13 +3387,7 @@ extern "C" int kifmm_plan_profile(kifmm_plan plan, int enable, double* phases) {
 extern "C" int kifmm_plan_check(kifmm_plan plan) {
     clear_error();
     KF_ARG(plan, "NULL plan");
-    int h = 0;
-    KF_CHECK_CUDA(cudaMemcpy(&h, plan->P.err.p, sizeof(int), cudaMemcpyDeviceToHost));
-    if (h) {
-        set_error("a tensor-core translation GEMM gave up waiting on its pipeline (code %d)", h);
-        return KIFMM_ERR_TIMEOUT;
-    }
-    return KIFMM_OK;
+    return check_waits(plan->P.err.p, 0);
 }
 
 extern "C" int kifmm_plan_destroy(kifmm_plan plan) {

@@ -3,6 +3,8 @@ instructions gives up as a whole or not at all."""
 import ctypes
 import os
 import re
+import subprocess
+import sys
 
 import pytest
 import torch
@@ -41,3 +43,40 @@ def test_a_warp_gives_up_as_a_whole(parity, raised, want):
     torch.cuda.synchronize()
     assert device_probe.lib().probe_wait_warp(ctypes.c_void_p(par.data_ptr()), raised, ctypes.c_void_p(got.data_ptr())) == 0
     assert got.tolist() == [want] * 32
+
+
+# A stand-in for the evaluation rows' launch: its wait gave up, and nothing was written.
+FAKE = """
+#include "%s/sliced.cuh"
+namespace kifmm {
+template <>
+int launch_sliced_store<float>(const SlicedTable&, int, const int4*, int, const int*, const int*, const __half*,
+                               const int*, const double*, float*, int, int* err, cudaStream_t s) {
+    return cudaMemsetAsync(err, 1, 1, s) == cudaSuccess ? KIFMM_OK : KIFMM_ERR_CUDA;
+}
+}
+"""
+
+CHILD = """
+import ctypes, sys
+ctypes.CDLL(sys.argv[1], ctypes.RTLD_GLOBAL)      # before the library, so that its call comes here
+import torch
+from paper_1605_01715_gb300 import KifmmError, Plan, Tree
+tree = Tree(torch.rand(3, 500, dtype=torch.float64, device="cuda"), max_leaf=32)
+try:
+    Plan(tree, kernel="sl", p=4, precision="mixed")
+    print("plan made")
+except KifmmError as e:
+    print(e.status)
+"""
+
+
+@pytest.mark.gpu
+def test_setup_reports_a_wait_that_gave_up(tmp_path):
+    from paper_1605_01715_gb300 import build as kb
+    src, so = tmp_path / "fake.cu", tmp_path / "fake.so"
+    src.write_text(FAKE % CSRC)
+    subprocess.run([kb.NVCC, "-shared", *kb.FLAGS, "-o", str(so), str(src)], check=True)
+    r = subprocess.run([sys.executable, "-c", CHILD, str(so)], capture_output=True, text=True, cwd=os.path.dirname(kb.HERE),
+                       timeout=300)
+    assert r.stdout.strip() == "TIMEOUT", r.stdout + r.stderr
