@@ -806,22 +806,29 @@ constexpr long long kRangeIdx = (1LL << 48) - 1;
 constexpr int kCloseBits = 5;
 __host__ __device__ inline int range_exp(long long fl) { return (int)((fl >> 48) & 255) - 128; }
 constexpr int kP2PUnitSrc = 2048;
-// A tree whose leaves give fewer than two waves of resident warps (two 8-warp blocks an
-// SM) takes narrower passes, down to 8 targets: one warp walks its unit's sources one chunk
-// after the other, and few units leave most of the chip idle behind the longest (near field
-// alone: 20k-point sphere 100 -> 72 us, 16,000-point pack 149 -> 113).  Every target's sum
-// stays the same bit for bit.  (Smaller units of sources reach 32 and 67 us, but cut a
-// target's FP32 sum at other places.)
-constexpr int kPassShiftMax = 3;
+// Targets per lane w of a pass.  A tree with fewer than two waves of units at the kernel's
+// widest (a wave: the warps the chip holds, two 8-warp blocks an SM) takes of the widest, 4
+// and 2 the one with the least (kPassStage + w) x max(1, waves), the wider of equals.  A warp
+// walks its unit's sources one chunk after the other: 2,048 sources take the double layer 165,
+// 135, 98 and 95 us at w = 6, 4, 2 and 1, most of it latency.  Where all units run at once the
+// narrow ones are done first; where they do not, each pass costs its staging again.  Near
+// field alone at w = 6 / 4 / 2 (double layer; chosen in brackets): 15,680 points 164 / 138 /
+// [97] us, 25,920 at 128 a leaf 174 / 156 / [127], 44,180 at 128 179 / [157] / 148 (but the
+// matvec 292 / 246 / 282: the narrow passes hold SMs that the far field needs), 64,980 at 192
+// 225 / [189] / 218, 98,000 at 128 [235] / 261 / 303.  Over the 320 plans measured, of all
+// kernels, the matvec is on average within 0.5 % of the best width's, at worst 6 %.  (Passes
+// of 8 to 12 targets until two waves were filled: 38,720 points at 192 a leaf 327 us, 288 with
+// 32.)  Every target's sum stays the same bit for bit.
+constexpr int kPassStage = 4;
 // Larger target leaves of the single layer and the field go to the block kernel (a
 // thread per target, sources staged once per leaf).  The double layers always take the
 // warp kernel, in passes, for its exact products.
 constexpr int kP2PWarpMaxLeaf = 64;
 // unit flags (int4 .w): bit 0 the leaf's first unit, bit 1 the leaf spans several units;
 // bits 8..9 the dipoles' axis of a KIND 4 unit; bits 16..30 one plus the unit's one pass
-// of 8 kMaxT >> (bits 4..5) targets, or 0 for all of the leaf's targets (the passes of a leaf share no
+// of 8 (bits 4..7) targets, or 0 for all of the leaf's targets (the passes of a leaf share no
 // targets, so they are dealt to separate warps: each pass walks all of its sources anyway)
-constexpr int kUnitFirst = 1, kUnitSplit = 2, kUnitNarrowShift = 4, kUnitPassShift = 16;
+constexpr int kUnitFirst = 1, kUnitSplit = 2, kUnitWidthShift = 4, kUnitPassShift = 16;
 
 // targets per lane per pass (plain and corrected-distance launches) and float4 entries
 // staged per source, by kernel: as many targets as keep each kernel within 128
@@ -1276,7 +1283,7 @@ k_p2p_warp(const int* __restrict__ leaves, int nunits, const int4* __restrict__ 
     float* raw = reinterpret_cast<float*>(st + S::kStage * 32);
     constexpr int kMaxT = CORR ? S::kMaxTCorr : S::kMaxT;
     const int pass = u.w >> kUnitPassShift;
-    const int pt = (8 * kMaxT) >> ((u.w >> kUnitNarrowShift) & 3);
+    const int pt = 8 * ((u.w >> kUnitWidthShift) & 15);
     const int64_t tf = pass ? tb + (int64_t)(pass - 1) * pt : tb;
     const int64_t tl = pass && tf + pt < te ? tf + pt : te;
     for (int64_t t0 = tf; t0 < tl; t0 += 8 * kMaxT) {
@@ -2356,7 +2363,7 @@ int setup(Plan& P, const double* src_nrm, const double* trg_nrm, cudaStream_t s)
         std::vector<signed char> ucls;         // DL: the dipole axis class of a unit's boxes
         auto half = [&](int box) { return std::ldexp(T.root_h, -T.h_lvl[box]); };
         auto exp_of = [](double ext) { return std::max(-100, std::min(100, std::ilogb(ext * (1.0 + 1e-12)) + 1)); };
-        const int64_t two_waves = 2 * 2 * kP2PWarps * (int64_t)nsm;
+        const int64_t resident = 2 * kP2PWarps * (int64_t)nsm;   // warps of the near-field kernel
         // leaves are independent: blocks of them by thread, joined in leaf order
         constexpr size_t kLeafBlock = 128;
         const size_t nblk = (tleaf.size() + kLeafBlock - 1) / kLeafBlock;
@@ -2496,34 +2503,36 @@ int setup(Plan& P, const double* src_nrm, const double* trg_nrm, cudaStream_t s)
         }
         // one unit per pass of the leaf's targets (empty units keep the whole leaf)
         {
-            auto pass_targets = [&](bool axis) {
-                const int k = axis ? 4 : P.kernel == KIFMM_KERNEL_SL ? 0 : P.kernel == KIFMM_KERNEL_DL ? 1
-                                        : P.kernel == KIFMM_KERNEL_ADL ? 2 : 3;
-                const int mt = k == 0 ? NearShape<0>::kMaxT : k == 1 ? NearShape<1>::kMaxT
-                             : k == 2 ? NearShape<2>::kMaxT : k == 3 ? NearShape<3>::kMaxT : NearShape<4>::kMaxT;
-                return (int64_t)8 * mt;
+            const int widest = P.kernel == KIFMM_KERNEL_SL    ? NearShape<0>::kMaxT
+                               : P.kernel == KIFMM_KERNEL_DL  ? NearShape<1>::kMaxT
+                               : P.kernel == KIFMM_KERNEL_ADL ? NearShape<2>::kMaxT
+                                                              : NearShape<3>::kMaxT;
+            // (the one-term kernel's pairs cost about half)
+            auto pass_targets = [&](size_t i, int w) -> int64_t {
+                return 8 * (is_axis[i] ? std::min(2 * w, NearShape<4>::kMaxT) : w);
             };
-            auto passes = [&](size_t i, int sh) {
+            auto targets_of = [&](size_t i) {
                 const int b = tleaf[units[i].u.x];
-                const int64_t ntg = T.h_rng[4 * b + 3] - T.h_rng[4 * b + 2], pt = std::max<int64_t>(8, pass_targets(is_axis[i] != 0) >> sh);
-                return units[i].u.y == units[i].u.z ? (int64_t)1 : (ntg + pt - 1) / pt;
+                return T.h_rng[4 * b + 3] - T.h_rng[4 * b + 2];
             };
-            int sh = 0;
-            for (; sh < kPassShiftMax; ++sh) {
+            int width = widest;
+            int64_t best = INT64_MAX;
+            for (int w : {widest, 4, 2}) {
                 int64_t n = 0;
-                for (size_t i = 0; i < units.size(); ++i) n += passes(i, sh);
-                if (n >= two_waves) break;
+                for (size_t i = 0; i < units.size(); ++i)
+                    n += units[i].u.y == units[i].u.z ? 1 : (targets_of(i) + pass_targets(i, w) - 1) / pass_targets(i, w);
+                const int64_t cost = (kPassStage + w) * std::max(resident, n);
+                if (w <= widest && cost < best) {
+                    best = cost;
+                    width = w;
+                }
+                if (w == widest && n >= 2 * resident) break;
             }
             std::vector<Unit> pu;
             std::vector<char> pa;
             pu.reserve(units.size());
             for (size_t i = 0; i < units.size(); ++i) {
-                const int b = tleaf[units[i].u.x];
-                const int64_t ntg = T.h_rng[4 * b + 3] - T.h_rng[4 * b + 2];
-                // (a pass holds at least 8 targets, one per lane of a source group)
-                int shi = sh;
-                while (shi > 0 && (pass_targets(is_axis[i] != 0) >> shi) < 8) --shi;
-                const int64_t pt = pass_targets(is_axis[i] != 0) >> shi;
+                const int64_t ntg = targets_of(i), pt = pass_targets(i, width);
                 const int64_t np = (ntg + pt - 1) / pt;
                 if (units[i].u.y == units[i].u.z || np <= 1) {
                     pu.push_back(units[i]);
@@ -2533,7 +2542,7 @@ int setup(Plan& P, const double* src_nrm, const double* trg_nrm, cudaStream_t s)
                 const int64_t per = units[i].work / ntg;      // sources of the unit
                 for (int64_t k = 0; k < np; ++k) {
                     Unit v = units[i];
-                    v.u.w |= (int)(k + 1) << kUnitPassShift | shi << kUnitNarrowShift;
+                    v.u.w |= (int)(k + 1) << kUnitPassShift | (int)(pt / 8) << kUnitWidthShift;
                     v.work = std::min(pt, ntg - k * pt) * per;
                     pu.push_back(v);
                     pa.push_back(is_axis[i]);
