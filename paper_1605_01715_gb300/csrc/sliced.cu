@@ -64,16 +64,6 @@ __global__ void __launch_bounds__(256) k_slice(const double* __restrict__ v, int
     }
 }
 
-// 1/sqrt(x) from the hardware's FP64 estimate y (its upper half: relative error below 2^-19)
-// and one step of Householder's third-order iteration, y (1 + e/2 + 3/8 e^2) with
-// e = 1 - x y^2, whose remainder 5/16 e^3 is below 2^-55.
-__device__ __forceinline__ double rsqrt3(double x) {
-    double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double e = fma(-(x * y), y, 1.0);
-    return fma(y * e, fma(0.375, e, 0.5), y);
-}
-
 // Nearest integer to x 2^(55 - e) (halves away from zero) for finite |x| < 2^e, from x's own
 // bits: the conversion would take the FP64 pipe.
 __device__ __forceinline__ long long fixed56(double x, int e) {
@@ -112,7 +102,7 @@ __global__ void __launch_bounds__(128) k_slice_eval(const int* __restrict__ tlea
         v[j] = 0.0;
         if (k < Q) {
             const double dx = x[0] - bpts[3 * k], dy = x[1] - bpts[3 * k + 1], dz = x[2] - bpts[3 * k + 2];
-            const double inv = rsqrt3(dx * dx + dy * dy + dz * dz);
+            const double inv = rsqrt(dx * dx + dy * dy + dz * dz);
             v[j] = grad ? (nv[0] * dx + nv[1] * dy + nv[2] * dz) * (inv * inv * inv) : inv;
         }
         top = max(top, (__double2hiint(v[j]) >> 20) & 0x7ff);

@@ -20,6 +20,7 @@
 namespace kifmm {
 
 constexpr int kSlices = 8;
+constexpr int kSliceBits = 7 * kSlices - 1;   // of the fixed point: the largest entry is below 2^kSliceBits
 constexpr int kSlicePairs = 64;         // columns (pairs) per tile
 constexpr int kSliceRows = 128;         // operator rows per work item
 
