@@ -737,9 +737,9 @@ def rooflines(phases, st, tst, args, kernel, peaks):
                       "peak_source": "%s bf16/fp16 dense burst %.0f / 3 (hi*hi + hi*lo + lo*hi)"
                                      % (src, pk["bf16_tflops"])}
     else:
-        peak = pk["bf16_tflops"] / 36.0             # FP64 products from 36 exact FP16 slice products
+        peak = pk["bf16_tflops"] / 45.0             # FP64 products from 45 exact FP16 slice products
         out["m2l"] = {"kernel": "k_sliced<double> (tcgen05, exact FP16 slices)", "bound": "tensor",
-                      "peak_source": "%s bf16/fp16 dense burst %.0f / 36 slice products" % (src, pk["bf16_tflops"])}
+                      "peak_source": "%s bf16/fp16 dense burst %.0f / 45 slice products" % (src, pk["bf16_tflops"])}
     out["m2l"].update({"achieved": flops / t / 1e12 if t > 0 else None, "peak": peak, "unit": "TFLOP/s",
                        "frac": flops / t / 1e12 / peak if t > 0 else None,
                        "traffic": _m2l_traffic(pairs, (ru + 15) // 16 * 16, (rd + 15) // 16 * 16) if mixed else None,

@@ -1908,8 +1908,8 @@ int check_waits(const int* err, cudaStream_t s) {
 // an FP64 product (W_d carries factors 1 / sigma, and its terms cancel to O(1)), rounded
 // once to FP32.  The kernel values of a chunk of targets are written as exact slices and
 // multiplied on the tensor cores (sliced.cuh): 98,000 targets at p = 10 took 21.7 ms as FP64
-// FMAs at the FP64 pipe's rate.  A chunk is 64 targets per SM: whole waves of the kernel, and
-// slices that stay in L2.
+// FMAs at the FP64 pipe's rate.  A chunk is one tile of targets per SM: whole waves of the
+// kernel, and slices that stay in L2.
 int build_d2t_sliced(Plan& P, const HostPinv& h, const std::vector<int>& tleaf_of, float* out, cudaStream_t s) {
     const Tree& T = P.tree->t;
     const int64_t nt = T.nt;

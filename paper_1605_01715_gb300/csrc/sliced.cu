@@ -19,12 +19,16 @@ constexpr int kOzABytes = kSliceRows * (int)kRowBytes;        // one slice of th
 constexpr int kOzBBytes = kSlicePairs * (int)kRowBytes;       // one slice of the inputs, one stage
 constexpr int kOzStageBytes = kSlices * (kOzABytes + kOzBBytes);
 constexpr int kOzSmemBytes = kOzStages * kOzStageBytes + 1024;
-constexpr int kOzChunk = 16;                                  // stages an accumulator stays exact over: 512 columns
+constexpr int kOzChunk = 14;                                  // stages an accumulator stays exact over: 448 columns
 constexpr int kOzWarps = 12, kOzThreads = kOzWarps * 32;
 constexpr int kOzProdWarp0 = 2, kOzProdThreads = 64;
 constexpr int kOzFoldWarp0 = 4, kOzFoldThreads = 256;
+constexpr int kOzFoldCols = kSlicePairs / 2;                  // columns of a fold warp
+static_assert(kSlices == 9 && kOzFoldCols % 8 == 0 && kSlicePairs % 16 == 0, "the copies' and folds' shares");
 static_assert(kOzStageBytes % 1024 == 0 && kOzSmemBytes <= 227 * 1024, "two stages fit");
-static_assert(kSlices * kSlicePairs == 512, "one accumulator per digit sum fills TMEM");
+static_assert(kSlices * kSlicePairs <= 512, "one accumulator per digit sum fits TMEM");
+static_assert((long long)kSlices * 64 * 64 * kOzChunk * kKS <= 1LL << 24, "accumulators stay exact");
+static_assert(kOzBBytes % 512 == 0 && kSlicePairs % 16 == 0, "slices of the inputs follow one another as rows of one operand");
 
 // x 2^e
 __device__ __forceinline__ double scale2(double x, int e) {
@@ -55,7 +59,7 @@ __global__ void __launch_bounds__(256) k_slice(const double* __restrict__ v, int
     if (lane == 0) exps[b] = fin ? e : kNotFinite;
     for (int k = lane; k < Kc; k += 32) {
         __half d[kSlices];
-        slice_digits(fin && k < K ? __double2ll_rn(scale2(x[k], 55 - e)) : 0LL, d);
+        slice_digits(fin && k < K ? __double2ll_rn(scale2(x[k], kSliceBits - e)) : 0LL, d);
 #pragma unroll
         for (int s = 0; s < kSlices; ++s) {
             if (PLANES) out[(size_t)s * plane + (size_t)b * Kc + k] = d[s];
@@ -64,14 +68,14 @@ __global__ void __launch_bounds__(256) k_slice(const double* __restrict__ v, int
     }
 }
 
-// Nearest integer to x 2^(55 - e) (halves away from zero) for finite |x| < 2^e, from x's own
-// bits: the conversion would take the FP64 pipe.
-__device__ __forceinline__ long long fixed56(double x, int e) {
+// Nearest integer to x 2^(kSliceBits - e) (halves away from zero) for finite |x| < 2^e, from
+// x's own bits: the conversion would take the FP64 pipe.
+__device__ __forceinline__ long long fixed_point(double x, int e) {
     const long long u = __double_as_longlong(x);
     const int ex = (int)((u >> 52) & 0x7ff);
-    if (ex == 0) return x == 0.0 ? 0LL : __double2ll_rn(scalbn(x, 55 - e));      // subnormal
+    if (ex == 0) return x == 0.0 ? 0LL : __double2ll_rn(scalbn(x, kSliceBits - e));      // subnormal
     const long long m = (u & 0xfffffffffffffLL) | 0x10000000000000LL;       // x = m 2^(ex - 1075)
-    const int sh = ex - 1075 + 55 - e;                                      // at most 2
+    const int sh = ex - 1075 + kSliceBits - e;                              // at most 9
     long long y = sh >= 0 ? m << sh : (sh > -64 ? ((m >> (-sh - 1)) + 1) >> 1 : 0LL);
     return u < 0 ? -y : y;
 }
@@ -120,45 +124,45 @@ __global__ void __launch_bounds__(128) k_slice_eval(const int* __restrict__ tlea
     for (int j = 0; j < NV; ++j) {
         if (j * 32 >= Kc) break;
         __half d[kSlices];
-        slice_digits(fin ? fixed56(v[j], e) : 0LL, d);
+        slice_digits(fin ? fixed_point(v[j], e) : 0LL, d);
 #pragma unroll
         for (int s = 0; s < kSlices; ++s) o[(size_t)j * 32 * kSlices + s * 32] = d[s];
     }
 }
 
-template <int COLS>
 __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t* r) {
-    static_assert(COLS == 8, "");
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
                  : "r"(taddr));
 }
 
-// The eight digit sums (exact integers in FP32) as one double, sum_d acc_d 128^-d: two
-// 64-bit integers of 46 bits, each made a double by placing it in the mantissa of a number
-// whose last place has its weight (2^-21, 2^-49), and one add.  Three FP64 adds in all.
+// The nine digit sums (exact integers in FP32) as one double, sum_d acc_d 128^-d: two
+// 64-bit integers below 2^51, each made a double by placing it in the mantissa of a number
+// whose last place has its weight (2^-28, 2^-56), and one add.  Three FP64 adds in all.
 __device__ __forceinline__ double join_digits(const uint32_t (&v)[kSlices][8], int c) {
+    static_assert(kSlices == 9, "digits 0 to 4 and 5 to 8");
     long long h = 0, l = 0;
 #pragma unroll
-    for (int d = 0; d < 4; ++d) {
-        h = h * 128 + __float2int_rn(__uint_as_float(v[d][c]));
-        l = l * 128 + __float2int_rn(__uint_as_float(v[4 + d][c]));
-    }
-    const double ch = 0x1.8p31, cl = 0x1.8p3;
+    for (int d = 0; d < 5; ++d) h = h * 128 + __float2int_rn(__uint_as_float(v[d][c]));
+#pragma unroll
+    for (int d = 5; d < 9; ++d) l = l * 128 + __float2int_rn(__uint_as_float(v[d][c]));
+    const double ch = 0x1.8p24, cl = 0x1.8p-4;
     return (__longlong_as_double(__double_as_longlong(ch) + h) - ch) + (__longlong_as_double(__double_as_longlong(cl) + l) - cl);
 }
 
 // STORE: write Real(oscale * value) (zeros in rows M .. ostride); else add into doubles.
 // Persistent over items (tile, group of 128 rows).  Warp 0: TMA of the operator slices;
-// warp 1: the 72 MMAs of a stage (36 slice pairs x 2 K steps), issued by an elected lane;
-// warps 2-3: cp.async of the gathered input slices; warps 4-11: digit sums to FP64 and out.
-// A stage's MMAs (128 x 64 x 16 each) take about 3.5 k clk for 262,144 FP64 products, 38
-// times the FP64 pipe's 2 a clock; its 96 KB of operands about as long to arrive.  Joining
-// the digit sums (three FP64 adds and a product per output) is not overlapped: about a
-// quarter of an item at K = 512.
-// 46,080-point sphere at p = 12 (K = 728, 80,360 V pairs): M2L 89.0 -> 3.44 ms, U2U and L2L
-// 29.9 -> 0.29 ms each against FP64 FMAs; the matvec's result differs by 2.4e-16.
-// Evaluation rows of 98,000 targets at p = 10 (with their slicing): 21.7 -> 3.5 ms.
+// warp 1: the MMAs of a stage (45 slice products x 2 K steps in 26 MMAs of 48 to 240 columns),
+// issued by an elected lane; warps 2-3: cp.async of the gathered input slices; warps 4-11: digit
+// sums to FP64 and out.
+// What bounds it: a stage takes 3.7 k clk with its share of the joins, 27 B a clock and SM of its
+// 99 KB of operands, the L2 fabric's rate as in the translation kernel; its MMAs are 2.2 k at the
+// tensor core's rate (one MMA a slice product would read A 45 times a K step instead of 13).  Tiles are 48 columns wide because nine
+// accumulators fill tensor memory's 512.  Joining the digit sums (three FP64 adds and a product
+// per output) is not overlapped.
+// 46,080-point sphere at p = 12 (K = 728, 80,360 V pairs): M2L 89.0 ms in FP64 FMAs, 3.44 with
+// eight slices in narrow MMAs, 3.08 so; U2U and L2L 29.9, 0.29 and 0.23 ms each.  Evaluation rows of
+// 98,000 targets at p = 10 (with their slicing): 21.7, 2.9 and 2.8 ms.
 template <typename Real, bool STORE>
 __global__ void __launch_bounds__(kOzThreads, 1)
 k_sliced(const __grid_constant__ CUtensorMap map, int64_t plane_rows, const int* __restrict__ aexp, int M, int Mr,
@@ -228,10 +232,11 @@ k_sliced(const __grid_constant__ CUtensorMap map, int64_t plane_rows, const int*
             }
         }
     } else if (warp == 1) {
-        // ---- MMA issue: slice pairs (i, j) with i + j <= 7 into accumulator i + j ----
+        // ---- MMA issue: slice pairs (i, j) with i + j <= 8 into accumulator i + j.  Slices j
+        // of the inputs follow one another in shared memory and accumulators i + j in tensor
+        // memory, so slice i of the operator takes its 9 - i partners in one or two wide MMAs ----
         const bool leader = elect_one();
         const uint64_t d0 = smem_desc(stage(0));
-        constexpr uint32_t idesc = idesc_f16(128, kSlicePairs);
         bool ok = true;
         int g = 0, f = 0;
         for (int k = 0; k < K && ok; ++k)
@@ -253,12 +258,15 @@ k_sliced(const __grid_constant__ CUtensorMap map, int64_t plane_rows, const int*
 #pragma unroll
                         for (int ks = 0; ks < 2; ++ks)
 #pragma unroll
-                            for (int a = 0; a < kSlices; ++a)
+                            for (int a = 0; a < kSlices; ++a) {
+                                const int nb = kSlices - a, w = nb > 5 ? (nb + 1) / 2 : nb;   // N <= 256
 #pragma unroll
-                                for (int b = 0; b < kSlices - a; ++b)
+                                for (int b = 0; b < nb; b += w)
                                     mma_f16(tmem + (uint32_t)((a + b) * kSlicePairs), a0 + a * (kOzABytes >> 4) + ks * 2,
-                                            b0 + b * (kOzBBytes >> 4) + ks * 2, idesc,
+                                            b0 + b * (kOzBBytes >> 4) + ks * 2,
+                                            idesc_f16(128, (b + w < nb ? w : nb - b) * kSlicePairs),
                                             (i == i0 && ks == 0 && a == 0) ? 0u : 1u);
+                            }
                         mma_commit(&empty[s]);
                         if (i == i1 - 1) mma_commit(&acc_full);
                     }
@@ -271,9 +279,10 @@ k_sliced(const __grid_constant__ CUtensorMap map, int64_t plane_rows, const int*
             if (!mbar_wait(&drain_bar, 0)) *abort = 1;
         }
     } else if (warp < kOzFoldWarp0) {
-        // ---- input slices by cp.async: a pair's 32 columns are 8 slices x 64 B in a row;
-        // thread pt copies 16-byte chunk pt % 32 of the 512 (slice chunk / 4) of pairs pt / 32 + 2 j ----
-        const int pt = tid - kOzProdWarp0 * 32, c = pt & 31, r0 = pt >> 5;
+        // ---- input slices by cp.async: a pair's 32 columns are 9 slices x 64 B in a row, 36
+        // chunks of 16 bytes.  Warp w copies pairs w, w + 2, ...: a chunk a lane of slices 0 to 7
+        // of one pair after the other, and slice 8 of eight pairs at a time ----
+        const int r0 = warp - kOzProdWarp0, cc = lane & 3, u = lane >> 2;
         int g = 0;
         bool ok = true;
         for (int k = 0; k < K && ok; ++k) {
@@ -288,14 +297,17 @@ k_sliced(const __grid_constant__ CUtensorMap map, int64_t plane_rows, const int*
                     ok = false;
                     break;
                 }
-                const uint32_t bs = stage(s) + (uint32_t)(kSlices * kOzABytes + (c >> 2) * kOzBBytes);
-#pragma unroll 8
-                for (int j = 0; j < kSlicePairs / 2; ++j) {
-                    const int bi = __shfl_sync(0xffffffffu, mine, j);
-                    const int row = r0 + 2 * j, cc = c & 3;
-                    const uint32_t o = (uint32_t)(row * (int)kRowBytes + ((cc ^ ((row >> 1) & 3)) << 4));
-                    const __half* src = in + ((size_t)(bi < 0 ? 0 : bi) * Kc + i * kKS) * kSlices + c * 8;
-                    cp_async16(bs + o, src, bi < 0 ? 0u : 16u);
+                const uint32_t bs = stage(s) + (uint32_t)(kSlices * kOzABytes);
+                auto copy = [&](int m, int slice) {        // this lane's chunk of the m-th pair's slice
+                    const int bi = __shfl_sync(0xffffffffu, mine, m);
+                    const __half* src = in + ((size_t)(bi < 0 ? 0 : bi) * Kc + i * kKS) * kSlices + slice * 32 + cc * 8;
+                    cp_async16(bs + (uint32_t)(slice * kOzBBytes) + sw64_off(r0 + 2 * m, cc), src, bi < 0 ? 0u : 16u);
+                };
+#pragma unroll
+                for (int m0 = 0; m0 < kSlicePairs / 2; m0 += 8) {
+#pragma unroll
+                    for (int m = m0; m < m0 + 8; ++m) copy(m, u);
+                    copy(m0 + u, 8);
                 }
                 cp_async_commit();
                 // the copies have landed before the next stage's begin: two stages hide it
@@ -305,17 +317,17 @@ k_sliced(const __grid_constant__ CUtensorMap map, int64_t plane_rows, const int*
             }
         }
     } else {
-        // ---- digit sums to FP64: lane quarter warp % 4, columns 32 half .. + 31 ----
+        // ---- digit sums to FP64: lane quarter warp % 4, columns 24 half .. + 23 ----
         const int quarter = warp & 3, half = (warp - kOzFoldWarp0) >> 2;
-        const uint32_t ta = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(half * 32);
+        const uint32_t ta = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(half * kOzFoldCols);
         int f = 0;
         for (int k = 0; k < K; ++k) {
             const int4 t = tiles[item(k) / mgroups];
             const int row = (item(k) % mgroups) * kSliceRows + quarter * 32 + lane;
             const int re = row < M ? aexp[(size_t)t.x * Mr + row] - 12 : 0;
-            double sum[32];
+            double sum[kOzFoldCols];
 #pragma unroll
-            for (int j = 0; j < 32; ++j) sum[j] = 0.0;
+            for (int j = 0; j < kOzFoldCols; ++j) sum[j] = 0.0;
             bool ok = true;
             for (int i0 = 0; i0 < nst; i0 += kOzChunk, ++f) {
                 if (!mbar_wait_warp(&acc_full, (uint32_t)(f & 1), abort)) {
@@ -324,12 +336,12 @@ k_sliced(const __grid_constant__ CUtensorMap map, int64_t plane_rows, const int*
                 }
                 tc_fence_after();
 #pragma unroll
-                for (int c0 = 0; c0 < 32; c0 += 8) {
+                for (int c0 = 0; c0 < kOzFoldCols; c0 += 8) {
                     uint32_t v[kSlices][8];
 #pragma unroll
-                    for (int d = 0; d < kSlices; ++d) tmem_ld8<8>(ta + (uint32_t)(d * kSlicePairs + c0), v[d]);
+                    for (int d = 0; d < kSlices; ++d) tmem_ld8(ta + (uint32_t)(d * kSlicePairs + c0), v[d]);
                     tmem_wait_ld();
-                    if (c0 == 24) {
+                    if (c0 + 8 == kOzFoldCols) {
                         tc_fence_before();
                         mbar_arrive(&acc_empty);
                     }
@@ -340,8 +352,8 @@ k_sliced(const __grid_constant__ CUtensorMap map, int64_t plane_rows, const int*
             if (!ok) break;
             if (row < (STORE ? ostride : M)) {
 #pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                    const int col = half * 32 + j;
+                for (int j = 0; j < kOzFoldCols; ++j) {
+                    const int col = half * kOzFoldCols + j;
                     if (col >= t.z) break;
                     const int ob = pout[t.y + col];
                     const int be = bexp[pin[t.y + col]];

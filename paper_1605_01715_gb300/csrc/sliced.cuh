@@ -1,15 +1,22 @@
 // FP64 products on the tensor cores from exact FP16 slices (the error-free splitting of
 // matrix products of Ozaki, Ogita, Oishi and Rump, Numerical Algorithms 59, 2012).
 //
-// A vector with |x| < 2^e is rounded once to the fixed point of 56 bits, x = 2^(e - 55) n,
-// and n written in balanced base-128 digits n = sum_s digit_s 128^(7 - s), digit_s in
-// [-64, 64]: eight FP16 slices of small integers.  A product of two vectors is then a sum
-// over slice pairs (i, j) of integer dot products.  Those with i + j <= 7 are kept, summed
-// by d = i + j: at most 8 pairs x 512 columns x 2^12 = 2^24, so eight FP32 accumulators of
-// the tensor core hold them exactly, whatever it does to bits below its last place.  The
-// accumulators are combined in 64-bit integers and two FP64 terms.  What is dropped is
-// below 2^-55 of (largest entry) x (largest entry) per column -- the order of FP64's own
-// rounding -- at 36 FP16 MMAs in place of FP64 FMAs (2 per clock and SM here).
+// A vector with |x| < 2^e is rounded once to the fixed point of 62 bits, x = 2^(e - 62) n:
+// exact for entries down to 2^-9 of the largest.  n is written in balanced base-128 digits
+// n = sum_s digit_s 128^(8 - s), digit_s in [-64, 64]: nine FP16 slices of small integers.  A
+// product of two vectors is then a sum over slice pairs (i, j) of integer dot products.  Those
+// with i + j <= 8 are kept, summed by d = i + j: at most 9 pairs x 448 columns x 2^12 < 2^24,
+// so nine FP32 accumulators of the tensor core hold them exactly, whatever it does to bits
+// below its last place.  The accumulators are combined in 64-bit integers and two FP64 terms.
+//
+// Error per column, for |a| < 2^ea and |b| < 2^eb: 2^-62 of 2^(ea + eb) from the fixed point,
+// and at most 1.008 x 2^-60 from the pairs left out (eight with i + j = 9 of 2^12 x 128^7 each,
+// over 2^124); each entry may be 2^(e - 1), so 2^-57.7 of the product of the largest entries.
+// FP64 products err by 2^-53 of each term and of each partial sum.  On the method's own
+// operators and check potentials (p = 3 to 10, all families) the error is at most 0.4 of that of
+// FP64 FMAs in order.  Eight slices with i + j <= 7 (at most 2^-51 per column) made up to 22 times
+// that error, where a row's largest entries meet the vector's smallest: neighbouring boxes of
+// the double layer at p = 6.  45 FP16 slice products in place of FP64 FMAs (2 per clock and SM here).
 #pragma once
 
 #include <cuda.h>
@@ -19,16 +26,16 @@
 
 namespace kifmm {
 
-constexpr int kSlices = 8;
+constexpr int kSlices = 9;
 constexpr int kSliceBits = 7 * kSlices - 1;   // of the fixed point: the largest entry is below 2^kSliceBits
-constexpr int kSlicePairs = 64;         // columns (pairs) per tile
+constexpr int kSlicePairs = 48;         // columns (pairs) per tile
 constexpr int kSliceRows = 128;         // operator rows per work item
 
 // Columns of a sliced vector: K rounded up to the 32 of a pipeline stage.
 inline int slice_cols(int K) { return (K + 31) / 32 * 32; }
 
 // Sliced operator tables: plane s holds digit s of every row (op * Mr + row), slice_cols(K)
-// wide, rows scaled by 2^(55 - exp); map: its TMA map over all planes.
+// wide, rows scaled by 2^(kSliceBits - exp); map: its TMA map over all planes.
 struct SlicedTable {
     DBuf<__half> planes;
     DBuf<int> exp;
@@ -41,7 +48,7 @@ struct SlicedTable {
 // Slice a row-major FP64 table of nops operators of Mr rows x K columns (row stride ld).
 int slice_table(const double* table, int64_t nops, int Mr, int K, int ld, SlicedTable& t, cudaStream_t s);
 
-// Slice vectors v[b][0..K) (stride ld) for b in [b0, b1): slices[b] holds slice_cols(K) x 8
+// Slice vectors v[b][0..K) (stride ld) for b in [b0, b1): slices[b] holds slice_cols(K) x 9
 // FP16 as [block of 32 columns][slice][32]; exps[b] = e (kNotFinite if an entry is not
 // finite: its products are NaN).
 constexpr int kNotFinite = -100000;
@@ -66,7 +73,7 @@ int slice_eval_rows(const int* tleaf_of, int64_t t0, int n, int64_t nt, const do
                     const int* lvl, const double* ctr, double root_h, const double* bpts, int Q, bool grad,
                     __half* slices, int* exps, double* oscale, cudaStream_t s);
 
-// Digits of y (|y| <= 2^55) in balanced base 128, most significant first.
+// Digits of y (|y| <= 2^62) in balanced base 128, most significant first.
 __device__ __forceinline__ void slice_digits(long long y, __half* d) {
 #pragma unroll
     for (int s = kSlices - 1; s > 0; --s) {

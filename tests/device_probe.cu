@@ -43,3 +43,27 @@ extern "C" int probe_eval_rows(const int* tleaf_of, int n, const double* txyz, c
                            oscale, 0));
     return cudaDeviceSynchronize() == cudaSuccess ? KIFMM_OK : KIFMM_ERR_CUDA;
 }
+
+// Slices the operators (nops of Mr rows x K, row stride ld) and vectors (nvec, stride vld),
+// both on the device, and multiplies the tiles' pairs (tiles: 4 ints each, on the host): added
+// into the doubles out, or with oscale stored as floats.
+extern "C" int probe_sliced_product(const double* table, int nops, int Mr, int K, int ld, int M, const double* vec, int nvec,
+                                    int vld, const int* tiles, int ntiles, const int* pin, const int* pout, void* out,
+                                    int ostride, const double* oscale, int* err) {
+    SlicedTable t;
+    DBuf<__half> sl;
+    DBuf<int> ex;
+    DBuf<int4> dt;
+    std::vector<int4> ht(ntiles);
+    for (int i = 0; i < ntiles; ++i) ht[i] = make_int4(tiles[4 * i], tiles[4 * i + 1], tiles[4 * i + 2], tiles[4 * i + 3]);
+    KF_TRY(slice_table(table, nops, Mr, K, ld, t, 0));
+    KF_TRY(sl.alloc((size_t)nvec * slice_cols(K) * kSlices));
+    KF_TRY(ex.alloc(nvec));
+    KF_TRY(dt.upload(ht, 0));
+    KF_TRY(slice_vectors(vec, K, vld, 0, nvec, sl.p, ex.p, 0));
+    if (oscale)
+        KF_TRY(launch_sliced_store<float>(t, M, dt.p, ntiles, pin, pout, sl.p, ex.p, oscale, (float*)out, ostride, err, 0));
+    else
+        KF_TRY(launch_sliced_add(t, M, dt.p, ntiles, pin, pout, sl.p, ex.p, (double*)out, ostride, err, 0));
+    return cudaDeviceSynchronize() == cudaSuccess ? KIFMM_OK : KIFMM_ERR_CUDA;
+}
