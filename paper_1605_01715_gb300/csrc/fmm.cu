@@ -2571,6 +2571,7 @@ int setup(Plan& P, const double* src_nrm, const double* trg_nrm, cudaStream_t s)
         KF_TRY(P.p2p_cranges.upload(hcr, s));
         P.n_p2p_units = (int)hu.size();
         P.n_p2p_corr = (int)hcu.size();
+        P.near_resident = resident;
         for (int k = 0; k < 5; ++k) KF_TRY(set_p2p_smem(k));
     }
     KF_TRY(stamp(1));
@@ -2735,13 +2736,8 @@ int run_pairs(const Plan& P, int which, const PairTiles& pt, int t0, int t1, con
 // (the 1M cube at 128 points per leaf: 52, once its exact zeros are left out; at 192:
 // 298; curved surfaces: several hundred).
 constexpr int64_t kLateNearPairs = 100;
-// Near-field pairs below which the far field's kernels are launched programmatically (each
-// one's prologue beside its predecessor's end): 20k sphere 139 -> 112 us, 2k sphere 57 -> 50.
-// The waiting blocks of the translation kernel hold whole SMs, which a larger near field
-// would use (24-instance forest, 150M pairs: 569 -> 603 us; 1M cube 773 -> 807).
-constexpr int64_t kPdlPairs = 50000000;
-inline bool pdl_chain(const Plan& P) { return P.near_pairs < kPdlPairs; }
-// Near-field pairs from which the X list stays in the far field's chain.
+// Near-field pairs from which the X list stays in the far field's chain.  Beside it, 93 plans
+// below took 0.97 to 1.44 times less (8 % on average), 29 above 0.96 to 1.07 (0.6 %).
 constexpr int64_t kXBesidePairs = 300000000;
 
 // Mixed precision: two-term FP16 on the tensor cores (tcgen05), every translation
@@ -2758,7 +2754,7 @@ int run_pairs<float>(const Plan& P, int which, const PairTiles& pt, int t0, int 
     const int Mr = out_up ? o.Ku : o.Kd, M = out_up ? o.ru : o.rd;
     // split even without tiles: M2L reads the splits the upward pass leaves behind
     if (b1 > b0) {
-        KF_TRY(tc_box_split(z, r, K, b0, b1, P.vin_h.p, P.vin_l.p, P.bexp.p, pdl_chain(P), s));
+        KF_TRY(tc_box_split(z, r, K, b0, b1, P.vin_h.p, P.vin_l.p, P.bexp.p, P.pdl, s));
         ++launches;
     }
     if (t1 <= t0) return KIFMM_OK;
@@ -2775,7 +2771,7 @@ int run_pairs<float>(const Plan& P, int which, const PairTiles& pt, int t0, int 
         }
     }
     KF_TRY(launch_pair_tc(which, m[0], m[1], o.texp[which], M, Mr, K, Mr, pt.tiles.p + t0, t1 - t0, pt.pin.p,
-                          pt.pout.p, P.bexp.p, P.vin_h.p, P.vin_l.p, out, P.err.p, pdl_chain(P), s, kc));
+                          pt.pout.p, P.bexp.p, P.vin_h.p, P.vin_l.p, out, P.err.p, P.pdl, s, kc));
     ++launches;
     return KIFMM_OK;
 }
@@ -2791,7 +2787,7 @@ int project(const Plan& P, int fam, const PairTiles& pt, float* z, cudaStream_t 
     const CUtensorMap* m = o.tmaps[fam];
     KF_TRY(launch_pair_tc(3, m[0], m[1], o.texp[fam], M, Mr, Kp, Mr, pt.tiles.p, pt.ntiles, pt.pin.p, pt.pout.p,
                           fam == 3 ? P.sexp.p : P.xexp.p, fam == 3 ? P.sin_h.p : P.xin_h.p,
-                          fam == 3 ? P.sin_l.p : P.xin_l.p, z, P.err.p, pdl_chain(P), s));
+                          fam == 3 ? P.sin_l.p : P.xin_l.p, z, P.err.p, P.pdl, s));
     launches += 2;
     return KIFMM_OK;
 }
@@ -2899,6 +2895,12 @@ int matvec(Plan& P, const Bufs<Real>& B, const double* q, double* out, cudaStrea
     const bool dl = P.kernel == KIFMM_KERNEL_DL;
     // mixed DL: the FP32 remainders of the dipoles too (the near field's exact products)
     const bool dl_lo = dl && std::is_same<Real, float>::value;
+    if (std::is_same<Real, float>::value) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        KF_CHECK_CUDA(cudaStreamIsCapturing(s, &cap));
+        P.pdl = chain_early(cap == cudaStreamCaptureStatusActive, P.kernel, P.near_pairs, P.n_p2l > 0, P.n_p2p_units,
+                            P.near_resident);
+    }
     KF_TRY(mark(0));
     if (near_overlap) {
         KF_CHECK_CUDA(cudaEventRecord(P.ev_start, s));
@@ -3038,7 +3040,7 @@ int matvec(Plan& P, const Bufs<Real>& B, const double* q, double* out, cudaStrea
     KF_TRY(mark(6));
     if (P.n_tleaf) {
         for (int c = 0; c < P.nc; ++c) {
-            KF_TRY(launch_pdl(mixed && pdl_chain(P), k_d2t<Real>, (unsigned)P.n_tleaf, 128u, dw * sizeof(Real), s, P.tleaf.p, T.rng.p,
+            KF_TRY(launch_pdl(mixed && P.pdl, k_d2t<Real>, (unsigned)P.n_tleaf, 128u, dw * sizeof(Real), s, P.tleaf.p, T.rng.p,
                               B.d2t + (size_t)c * T.nt * dw, dn, dw, B.res + (size_t)c * T.nt));
             ++launches;
         }

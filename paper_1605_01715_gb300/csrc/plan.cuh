@@ -63,6 +63,22 @@ struct OpTables {
     }
 };
 
+// Whether the far field's kernels are launched programmatically, each one's prologue beside its
+// predecessor's end.  Launched one by one that also hides the gaps between launches: 57 plans of
+// all kernels below 50M near-field pairs are 0.84 to 1.35 times as fast with it (12 % on average;
+// without / with: 20k sphere 139 / 112 us, 26,000-point forest 273 / 202, 120,000-point cube 254 /
+// 213).  In a captured graph there are no such gaps, and the waiting blocks of the translation
+// kernel hold whole SMs that a near field of many pairs, or of more than a wave of units (resident:
+// the warps the chip holds) beside an X list, would use.  Of 380 such plans the 286 that take it
+// gain 3 % on average (at most 16), the others below 50M pairs would lose 7 % (at most 25): double
+// layer of 120,000 points 209 / 228 us, of 25,920 at 192 a leaf 183 / 223, single layer of 72,000
+// (33M pairs, 1.7 waves) 208 / 238, 64,000-point pack (41M, 1.5 waves) 303 / 354.
+inline bool chain_early(bool captured, int kernel, int64_t near_pairs, bool x_list, int64_t units, int64_t resident) {
+    const bool dl = kernel == KIFMM_KERNEL_DL;
+    if (!captured) return near_pairs < 50000000;
+    return near_pairs < (dl ? 20000000 : 50000000) && (near_pairs < 12000000 || 10 * units <= 11 * resident || (!dl && !x_list));
+}
+
 struct Plan {
     kifmm_tree_s* tree = nullptr;
     int kernel = 0, p = 0, Q = 0, Qp = 0, prec = 0;
@@ -107,6 +123,8 @@ struct Plan {
                                           // end range, flags: 1 first of its leaf, 2 leaf split)
     DBuf<longlong2> p2p_ranges;           // mixed: source index ranges of the units
     int n_p2p_units = 0, n_p2p_split = 0;
+    int64_t near_resident = 0;            // mixed: near-field warps the chip holds
+    bool pdl = false;                     // mixed: this matvec's far field launched early (chain_early)
     int64_t near_pairs = 0;               // mixed: (target, source) pairs the near field evaluates
     DBuf<int4> p2p_cunits;                // mixed: one unit per range with close pairs (the
     DBuf<longlong2> p2p_cranges;          //   corrected-distance launch) and those ranges

@@ -1,5 +1,6 @@
 // Kernels that run single device functions of the library, for tests (built by device_probe.py).
 #include "../paper_1605_01715_gb300/csrc/pair_tc.cuh"
+#include "../paper_1605_01715_gb300/csrc/plan.cuh"
 #include "../paper_1605_01715_gb300/csrc/sliced.cuh"
 
 using namespace kifmm;
@@ -66,4 +67,9 @@ extern "C" int probe_sliced_product(const double* table, int nops, int Mr, int K
     else
         KF_TRY(launch_sliced_add(t, M, dt.p, ntiles, pin, pout, sl.p, ex.p, (double*)out, ostride, err, 0));
     return cudaDeviceSynchronize() == cudaSuccess ? KIFMM_OK : KIFMM_ERR_CUDA;
+}
+
+extern "C" int probe_chain_early(int captured, int kernel, long long near_pairs, int x_list, long long units,
+                                 long long resident) {
+    return chain_early(captured != 0, kernel, near_pairs, x_list != 0, units, resident);
 }

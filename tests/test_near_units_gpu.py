@@ -43,3 +43,20 @@ def test_pass_width(kernel, p, freq, leaf):
         width = WIDEST[kernel]
     print(kernel, mesh.n, leaf, units, width)
     assert plan.stats()["near_units"] == units[width]
+
+
+@pytest.mark.parametrize("kernel,pairs,x_list,units,direct,captured", [
+    # plans timed with and without (2,432 resident warps)
+    ("dl", 3.6e6, 0, 628, True, True), ("sl", 11.1e6, 0, 2236, True, True), ("adl", 14.8e6, 1, 1348, True, True),
+    ("sl", 30.7e6, 1, 2072, True, True), ("dl", 11.6e6, 0, 3248, True, True), ("sl", 23.5e6, 0, 5816, True, True),
+    ("dl", 31.0e6, 0, 4864, True, False), ("sl", 32.6e6, 1, 4232, True, False), ("dl", 37.4e6, 0, 1784, True, False),
+    ("dl", 17.2e6, 1, 4880, True, False), ("adl", 40.9e6, 1, 3546, True, False), ("sl", 77.2e6, 1, 2440, False, False),
+    ("adl", 628.3e6, 1, 33792, False, False),
+])
+def test_early_launch_rule(kernel, pairs, x_list, units, direct, captured):
+    import ctypes
+    import device_probe
+    from paper_1605_01715_gb300.capi import KERNELS
+    f = device_probe.lib().probe_chain_early
+    f.argtypes = [ctypes.c_int, ctypes.c_int, ctypes.c_longlong, ctypes.c_int, ctypes.c_longlong, ctypes.c_longlong]
+    assert [bool(f(cap, KERNELS[kernel], int(pairs), x_list, units, 2432)) for cap in (0, 1)] == [direct, captured]
