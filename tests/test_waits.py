@@ -11,7 +11,7 @@ import torch
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1605_01715_gb300", "csrc")
 # a use of TMEM by a role of the kernels, and what makes a wait's outcome the warp's before it
-TMEM_USE = re.compile(r"\b(?:fold_acc<\w+>|tmem_ld8?<\w+>|tmem_st32)\(")
+TMEM_USE = re.compile(r"\b(?:fold_acc<\w+>|tmem_ld8?(?:<\w+>)?|tmem_st32)\(")
 WAIT = re.compile(r"\bmbar_wait(?:_ab|_warp)?\(")
 VOTE = re.compile(r"__all_sync\(|bar_named_or\(")
 
