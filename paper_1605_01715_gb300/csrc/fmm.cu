@@ -831,11 +831,14 @@ constexpr int kP2PWarpMaxLeaf = 64;
 constexpr int kUnitFirst = 1, kUnitSplit = 2, kUnitWidthShift = 4, kUnitPassShift = 16;
 
 // targets per lane per pass (plain and corrected-distance launches) and float4 entries
-// staged per source, by kernel: as many targets as keep each kernel within 128
-// registers, so two blocks share an SM (the double layer's 6 spill a little and still win:
-// staging a chunk of sources costs a pass about half of what its pairs do, and a leaf of 48
-// targets is one pass.  1M sphere, near field alone: 4 targets 1611 us, 5 1694, 6 1532, 8
-// 1549; the adjoint's 6 lose, 64-sphere pack 1027 -> 1063)
+// staged per source, by kernel: as many targets as keep each kernel within 128 registers, so
+// two blocks share an SM.  The double layer's 6 do not fit: 180 bytes of spill stores and 568 of
+// loads, one source in flight instead of two, offsets formed anew.  In trees of two waves and
+// more they win all the same, as staging a chunk of sources costs a pass about half of what its
+// pairs do and a leaf of 48 targets is one pass: 1M sphere, near field alone, 4 targets 1611 us,
+// 5 1694, 6 1532, 8 1549, 255,380 points at 96 a leaf 456 / 411 at 4 / 6; the 270,000-element
+// cube loses, 175 / 198, but its matvec, far field beside, does not, 398 / 390.  The adjoint's
+// 6 lose, 64-sphere pack 1027 -> 1063.
 template <int KIND> struct NearShape;
 template <> struct NearShape<0> { static constexpr int kMaxT = 8, kMaxTCorr = 6, kStage = 4, kRaw = 7; };
 template <> struct NearShape<1> { static constexpr int kMaxT = 6, kMaxTCorr = 4, kStage = 7, kRaw = 12; };
@@ -1731,7 +1734,7 @@ int translation_ops(const Plan& P, const HostPinv& h, int which, int C, int Kc, 
     rs.bset = dbs.p;
     rs.orow = dor.p;
     rs.bpts = db.p;
-    KF_TRY(build_rows<double>(rs, P.Q, C, Kc, dP, 0, out, s));
+    KF_TRY(build_rows(rs, P.Q, C, Kc, dP, 0, out, s));
     KF_CHECK_CUDA(cudaStreamSynchronize(s));   // the row descriptors are freed on return
     return KIFMM_OK;
 }
@@ -1990,7 +1993,7 @@ int build_d2t(Plan& P, const HostPinv& h, const std::vector<int>& tleaf_of, int 
         rs.bset = nullptr;
         rs.orow = orow.p + r0;
         rs.bpts = bpts.p;
-        KF_TRY(build_rows<double>(rs, P.Q, P.Q, P.Qp, dPd.p, adl ? 1 : 0, out, s));
+        KF_TRY(build_rows(rs, P.Q, P.Q, P.Qp, dPd.p, adl ? 1 : 0, out, s));
     }
     KF_CHECK_CUDA(cudaStreamSynchronize(s));
     return KIFMM_OK;
@@ -2722,22 +2725,23 @@ int setup(Plan& P, const double* src_nrm, const double* trg_nrm, cudaStream_t s)
 
 template <typename Real>
 struct Bufs {
-    const Real *m2m, *m2l, *l2l, *d2t, *surf, *tnrm;
+    const Real *d2t, *surf, *tnrm;
     Real *u, *d, *res, *q;
 };
 
 enum { kU2U = 0, kM2L = 1, kL2L = 2 };
 
 template <typename Real>
-int run_pairs(const Plan& P, int which, const PairTiles& pt, int t0, int t1, const Real* ops, const Real* in,
-              Real* out, int b0, int b1, cudaStream_t s, int& launches);
+int run_pairs(const Plan& P, int which, const PairTiles& pt, int t0, int t1, const Real* in, Real* out, int b0, int b1,
+              cudaStream_t s, int& launches);
 
 // Evaluated near-field pairs per target below which the near field starts after M2L
 // (the 1M cube at 128 points per leaf: 52, once its exact zeros are left out; at 192:
 // 298; curved surfaces: several hundred).
 constexpr int64_t kLateNearPairs = 100;
-// Near-field pairs from which the X list stays in the far field's chain.  Beside it, 93 plans
-// below took 0.97 to 1.44 times less (8 % on average), 29 above 0.96 to 1.07 (0.6 %).
+// Near-field pairs from which the X list stays in the far field's chain.  With it beside the
+// upward pass and M2L 93 plans below were 0.97 to 1.44 times as fast (8 % on average), 29 above
+// 0.96 to 1.07 times (0.6 %).
 constexpr int64_t kXBesidePairs = 300000000;
 
 // Mixed precision: two-term FP16 on the tensor cores (tcgen05), every translation
@@ -2745,9 +2749,8 @@ constexpr int64_t kXBesidePairs = 300000000;
 // Ku per box), M2L from the up to the down basis, L2L in the down basis (rd of Kd).
 // The input vectors of a launch (boxes [b0, b1)) are scaled and split first.
 template <>
-int run_pairs<float>(const Plan& P, int which, const PairTiles& pt, int t0, int t1, const float* ops,
-                     const float* z, float* out, int b0, int b1, cudaStream_t s, int& launches) {
-    (void)ops;  // the tensor-core path reads the split tables through their TMA maps
+int run_pairs<float>(const Plan& P, int which, const PairTiles& pt, int t0, int t1, const float* z, float* out,
+                     int b0, int b1, cudaStream_t s, int& launches) {
     const OpTables& o = *P.ops;
     const bool in_up = which != kL2L, out_up = which == kU2U;
     const int K = in_up ? o.Ku : o.Kd, r = in_up ? o.ru : o.rd;
@@ -2795,9 +2798,8 @@ int project(const Plan& P, int fam, const PairTiles& pt, float* z, cudaStream_t 
 // FP64: exact FP16 slices on the tensor cores (sliced.cuh); the inputs of the launch (boxes
 // [b0, b1)) are sliced first.
 template <>
-int run_pairs<double>(const Plan& P, int which, const PairTiles& pt, int t0, int t1, const double* ops,
-                      const double* in, double* out, int b0, int b1, cudaStream_t s, int& launches) {
-    (void)ops;
+int run_pairs<double>(const Plan& P, int which, const PairTiles& pt, int t0, int t1, const double* in, double* out,
+                      int b0, int b1, cudaStream_t s, int& launches) {
     if (b1 > b0) {
         KF_TRY(slice_vectors(in, P.Q, P.Qp, b0, b1, P.vsl.p, P.bexp.p, s));
         ++launches;
@@ -2889,8 +2891,8 @@ int matvec(Plan& P, const Bufs<Real>& B, const double* q, double* out, cudaStrea
         ++launches;
         return KIFMM_OK;
     };
-    // mixed, warp near field: it runs on its own stream beside the far field (forked
-    // after the gather) and the far field is added once both are done
+    // mixed: the near field runs on its own stream beside the far field (forked after the
+    // gather) and the far field is added once both are done
     const bool near_overlap = std::is_same<Real, float>::value && P.n_tleaf && P.near_stream && !P.serial;
     const bool dl = P.kernel == KIFMM_KERNEL_DL;
     // mixed DL: the FP32 remainders of the dipoles too (the near field's exact products)
@@ -3001,7 +3003,7 @@ int matvec(Plan& P, const Bufs<Real>& B, const double* q, double* out, cudaStrea
         KF_TRY(project(P, 3, P.proj_up, up, s, launches));
     }
     for (int l = T.nlev - 1; l >= 2; --l)
-        KF_TRY(run_pairs<Real>(P, kU2U, P.u2u, P.u2u.level_tile[l], P.u2u.level_tile[l + 1], B.m2m, up, up,
+        KF_TRY(run_pairs<Real>(P, kU2U, P.u2u, P.u2u.level_tile[l], P.u2u.level_tile[l + 1], up, up,
                                T.level_off[std::min(l + 1, T.nlev)], T.level_off[std::min(l + 2, T.nlev)], s,
                                launches));
     KF_TRY(mark(3));
@@ -3015,7 +3017,7 @@ int matvec(Plan& P, const Bufs<Real>& B, const double* q, double* out, cudaStrea
     }
     KF_TRY(mark(4));
     // the upward pass split levels 3 and deeper (mixed); level 2 is split here
-    KF_TRY(run_pairs<Real>(P, kM2L, P.m2l, 0, P.m2l.ntiles, B.m2l, up, dn, T.level_off[std::min(2, T.nlev)],
+    KF_TRY(run_pairs<Real>(P, kM2L, P.m2l, 0, P.m2l.ntiles, up, dn, T.level_off[std::min(2, T.nlev)],
                            T.level_off[std::min(3, T.nlev)], s, launches));
     if (late_near) {
         KF_CHECK_CUDA(cudaEventRecord(P.ev_fork, s));
@@ -3028,7 +3030,7 @@ int matvec(Plan& P, const Bufs<Real>& B, const double* q, double* out, cudaStrea
     const bool center = !mixed && gradient_kernel(P.kernel);
     for (int l = 2; l < T.nlev; ++l) {
         if (l >= 3)
-            KF_TRY(run_pairs<Real>(P, kL2L, P.l2l, P.l2l.level_tile[l], P.l2l.level_tile[l + 1], B.l2l, dn, dn,
+            KF_TRY(run_pairs<Real>(P, kL2L, P.l2l, P.l2l.level_tile[l], P.l2l.level_tile[l + 1], dn, dn,
                                    T.level_off[l - 1], T.level_off[l], s, launches));
         int nl = T.level_off[l + 1] - T.level_off[l];
         if (center && nl > 0) {
@@ -3080,12 +3082,10 @@ int matvec(Plan& P, const Bufs<Real>& B, const double* q, double* out, cudaStrea
 
 int plan_matvec(Plan& P, const double* q, double* out, cudaStream_t s) {
     if (P.fp64) {
-        Bufs<double> B{nullptr, nullptr, nullptr, P.d2t_d.p, P.surf_d.p, P.tnrm_d.p,
-                       P.u_d.p,   P.d_d.p,   P.res_d.p, P.q_d.p};
+        Bufs<double> B{P.d2t_d.p, P.surf_d.p, P.tnrm_d.p, P.u_d.p, P.d_d.p, P.res_d.p, P.q_d.p};
         return matvec<double>(P, B, q, out, s);
     }
-    Bufs<float> B{nullptr, nullptr, nullptr, P.d2t_f.p, P.surf_f.p, P.tnrm_f.p,
-                  P.u_f.p,   P.d_f.p,   P.res_f.p, P.q_f.p};
+    Bufs<float> B{P.d2t_f.p, P.surf_f.p, P.tnrm_f.p, P.u_f.p, P.d_f.p, P.res_f.p, P.q_f.p};
     return matvec<float>(P, B, q, out, s);
 }
 

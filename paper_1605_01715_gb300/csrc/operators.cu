@@ -263,11 +263,10 @@ void up_skeleton(const UpPivots& f, int k, std::vector<int>& idx, std::vector<do
 // out[orow[r]*Cp + j] = ascale[r] * sum_m G(a_r, b_{bset[r], m}) P[m][j],  j < C; 0 for C <= j < Cp
 // (P is Q x C: the Q points of a b set by C columns)
 // G = 1/|a-b| (kfun 0) or n_r.(a-b)/|a-b|^3 (kfun 1).  8 rows per block.
-template <typename Real>
 __global__ void k_build_rows(int nrows, const double* __restrict__ apts, const double* __restrict__ anrm,
                              const double* __restrict__ ascale, const int* __restrict__ bset,
                              const int64_t* __restrict__ orow, const double* __restrict__ bpts, int Q,
-                             int C, int Cp, const double* __restrict__ P, int kfun, Real* __restrict__ out) {
+                             int C, int Cp, const double* __restrict__ P, int kfun, double* __restrict__ out) {
     extern __shared__ double Ks[];  // [8][Q]
     const int R = 8;
     int r0 = blockIdx.x * R;
@@ -304,28 +303,24 @@ __global__ void k_build_rows(int nrows, const double* __restrict__ apts, const d
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             int row = r0 + r;
-            if (row < nrows) out[(size_t)orow[row] * Cp + j] = (Real)(ascale[row] * acc[r]);
+            if (row < nrows) out[(size_t)orow[row] * Cp + j] = ascale[row] * acc[r];
         }
     }
 }
 
-template <typename Real>
-int build_rows(const RowSpec& rs, int Q, int C, int Cp, const double* dP, int kfun, Real* out,
+int build_rows(const RowSpec& rs, int Q, int C, int Cp, const double* dP, int kfun, double* out,
                cudaStream_t s) {
     if (rs.nrows == 0) return KIFMM_OK;
     size_t smem = 8 * (size_t)Q * sizeof(double);
     if (smem > 48 * 1024)
-        KF_CHECK_CUDA(cudaFuncSetAttribute(k_build_rows<Real>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        KF_CHECK_CUDA(cudaFuncSetAttribute(k_build_rows, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            (int)smem));
-    k_build_rows<Real><<<div_up(rs.nrows, 8), 256, smem, s>>>(rs.nrows, rs.apts, rs.anrm, rs.ascale,
+    k_build_rows<<<div_up(rs.nrows, 8), 256, smem, s>>>(rs.nrows, rs.apts, rs.anrm, rs.ascale,
                                                               rs.bset, rs.orow, rs.bpts, Q, C, Cp, dP, kfun,
                                                               out);
     KF_CHECK_LAUNCH();
     return KIFMM_OK;
 }
-
-template int build_rows<float>(const RowSpec&, int, int, int, const double*, int, float*, cudaStream_t);
-template int build_rows<double>(const RowSpec&, int, int, int, const double*, int, double*, cudaStream_t);
 
 // Host-side row descriptors of the three translation-operator tables.
 void translation_rows(const HostPinv& h, int which, std::vector<double>& apts, std::vector<int>& bset,

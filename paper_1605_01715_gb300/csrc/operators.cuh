@@ -67,8 +67,7 @@ struct RowSpec {
     const double* bpts = nullptr;    // sets of Q points, 3 doubles each
 };
 
-template <typename Real>
-int build_rows(const RowSpec& rs, int Q, int C, int Cp, const double* dP, int kfun, Real* out, cudaStream_t s);
+int build_rows(const RowSpec& rs, int Q, int C, int Cp, const double* dP, int kfun, double* out, cudaStream_t s);
 
 // which: 0 = M2M', 1 = M2L', 2 = L2L'
 void translation_rows(const HostPinv& h, int which, std::vector<double>& apts, std::vector<int>& bset,

@@ -245,9 +245,11 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
 // COLS consecutive TMEM columns of the warp's 32 lanes into registers (one column each).
 template <int COLS>
 __device__ __forceinline__ void tmem_ld(uint32_t taddr, uint32_t* r) {
-    static_assert(COLS == 16 || COLS == 32 || COLS == 64, "one load instruction");
+    static_assert(COLS == 8 || COLS == 16 || COLS == 32 || COLS == 64, "one load instruction");
 #define KF_R8(o) "=r"(r[o]), "=r"(r[o + 1]), "=r"(r[o + 2]), "=r"(r[o + 3]), "=r"(r[o + 4]), "=r"(r[o + 5]), "=r"(r[o + 6]), "=r"(r[o + 7])
-    if constexpr (COLS == 16) {
+    if constexpr (COLS == 8) {
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];" : KF_R8(0) : "r"(taddr));
+    } else if constexpr (COLS == 16) {
         asm volatile(
             "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
             "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"

@@ -33,13 +33,13 @@ struct BieScratch {
 };
 
 // Translation tables of one (device, order, cutoffs, precision, ADL centring): shared by
-// every plan with that key, freed with the last of them.  FP64 form: m2m/m2l/l2l in
-// FP64, Qp x Qp each.  Mixed form: every translation acts between projections onto
-// the ranges of the pseudo-inverses (P = W U^T, U orthonormal): families 0 M2M''
-// = U_u^T M2M' W_u (Ku x Ku), 1 M2L'' = U_d^T M2L' W_u (Kd x Ku), 2 L2L'' = U_d^T
-// L2L' W_d (Kd x Kd), and the projections 3 U_u^T and 4 U_d^T (K x Qp), as FP16 hi/lo
-// tables scaled by 2^texp, with their TMA tensor maps.  ru / rd: the ranks, Ku / Kd:
-// rounded up to 16.
+// every plan with that key, freed with the last of them.  FP64 form: M2M', M2L' and L2L',
+// Q x Q each, as exact slices (sliced.cuh; 18 bytes an entry, and while they are built the FP64
+// tables' 8 beside them).  Mixed form: every translation acts between projections onto the
+// ranges of the pseudo-inverses (P = W U^T, U orthonormal): families 0 M2M'' = U_u^T M2M' W_u
+// (Ku x Ku), 1 M2L'' = U_d^T M2L' W_u (Kd x Ku), 2 L2L'' = U_d^T L2L' W_d (Kd x Kd), and the
+// projections 3 U_u^T and 4 U_d^T (K x Qp), as FP16 hi/lo tables scaled by 2^texp, with their
+// TMA tensor maps.  ru / rd: the ranks, Ku / Kd: rounded up to 16.
 constexpr int kFamilies = 5;
 struct OpTables {
     int device = 0, p = 0;
@@ -50,7 +50,7 @@ struct OpTables {
     int ru = 0, rd = 0, Ku = 0, Kd = 0;
     int ks = 0;                     // mixed: S2U points (skeleton of the up-check surface)
     DBuf<float> surf_up;            // mixed: those points on the unit surface, ks x 3
-    SlicedTable fp64_ops[3];        // FP64: M2M', M2L', L2L' in exact slices (see sliced.cuh)
+    SlicedTable fp64_ops[3];        // FP64: M2M', M2L', L2L'
     SlicedTable wd;                 // mixed: W_d^T (rd of Kd rows), the evaluation rows' factor
     DBuf<__half> tab_h[kFamilies], tab_l[kFamilies];
     int texp[kFamilies] = {0, 0, 0, 0, 0};

@@ -130,12 +130,6 @@ __global__ void __launch_bounds__(128) k_slice_eval(const int* __restrict__ tlea
     }
 }
 
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t* r) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                 : "r"(taddr));
-}
-
 // The nine digit sums (exact integers in FP32) as one double, sum_d acc_d 128^-d: two
 // 64-bit integers below 2^51, each made a double by placing it in the mantissa of a number
 // whose last place has its weight (2^-28, 2^-56), and one add.  Three FP64 adds in all.
@@ -339,7 +333,7 @@ k_sliced(const __grid_constant__ CUtensorMap map, int64_t plane_rows, const int*
                 for (int c0 = 0; c0 < kOzFoldCols; c0 += 8) {
                     uint32_t v[kSlices][8];
 #pragma unroll
-                    for (int d = 0; d < kSlices; ++d) tmem_ld8(ta + (uint32_t)(d * kSlicePairs + c0), v[d]);
+                    for (int d = 0; d < kSlices; ++d) tmem_ld<8>(ta + (uint32_t)(d * kSlicePairs + c0), v[d]);
                     tmem_wait_ld();
                     if (c0 + 8 == kOzFoldCols) {
                         tc_fence_before();
@@ -438,7 +432,5 @@ int launch_sliced_store(const SlicedTable& t, int M, const int4* tiles, int ntil
 }
 template int launch_sliced_store<float>(const SlicedTable&, int, const int4*, int, const int*, const int*, const __half*,
                                         const int*, const double*, float*, int, int*, cudaStream_t);
-template int launch_sliced_store<double>(const SlicedTable&, int, const int4*, int, const int*, const int*,
-                                         const __half*, const int*, const double*, double*, int, int*, cudaStream_t);
 
 }  // namespace kifmm

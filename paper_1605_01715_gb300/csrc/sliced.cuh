@@ -56,7 +56,7 @@ int slice_vectors(const double* v, int K, int ld, int b0, int b1, __half* slices
 
 // out[pout[j]][row] (+)= sum_k Op[row][k] in[pin[j]][k] for every pair of the tiles (op,
 // first pair, pairs <= kSlicePairs, 0), rows < M.  FP64: added by atomics into ostride
-// doubles per output.  FP32 / FP64 store: written, times oscale[pout[j]], with zeros in
+// doubles per output.  FP32 store: written, times oscale[pout[j]], with zeros in
 // rows M..ostride.  err: a word a wait that gave up sets.
 int launch_sliced_add(const SlicedTable& t, int M, const int4* tiles, int ntiles, const int* pin, const int* pout,
                       const __half* in, const int* exps, double* out, int ostride, int* err, cudaStream_t s);
