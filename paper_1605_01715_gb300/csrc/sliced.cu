@@ -19,7 +19,7 @@ constexpr int kOzABytes = kSliceRows * (int)kRowBytes;        // one slice of th
 constexpr int kOzBBytes = kSlicePairs * (int)kRowBytes;       // one slice of the inputs, one stage
 constexpr int kOzStageBytes = kSlices * (kOzABytes + kOzBBytes);
 constexpr int kOzSmemBytes = kOzStages * kOzStageBytes + 1024;
-constexpr int kOzChunk = 14;                                  // stages an accumulator stays exact over: 448 columns
+constexpr int kOzChunk = 16;                                  // stages accumulators 0 to 7 stay exact over: 512 columns
 constexpr int kOzWarps = 12, kOzThreads = kOzWarps * 32;
 constexpr int kOzProdWarp0 = 2, kOzProdThreads = 64;
 constexpr int kOzFoldWarp0 = 4, kOzFoldThreads = 256;
@@ -27,7 +27,7 @@ constexpr int kOzFoldCols = kSlicePairs / 2;                  // columns of a fo
 static_assert(kSlices == 9 && kOzFoldCols % 8 == 0 && kSlicePairs % 16 == 0, "the copies' and folds' shares");
 static_assert(kOzStageBytes % 1024 == 0 && kOzSmemBytes <= 227 * 1024, "two stages fit");
 static_assert(kSlices * kSlicePairs <= 512, "one accumulator per digit sum fits TMEM");
-static_assert((long long)kSlices * 64 * 64 * kOzChunk * kKS <= 1LL << 24, "accumulators stay exact");
+static_assert((long long)(kSlices - 1) * 64 * 64 * kOzChunk * kKS <= 1LL << 24, "all accumulators but the last stay exact");
 static_assert(kOzBBytes % 512 == 0 && kSlicePairs % 16 == 0, "slices of the inputs follow one another as rows of one operand");
 
 // x 2^e
@@ -130,7 +130,7 @@ __global__ void __launch_bounds__(128) k_slice_eval(const int* __restrict__ tlea
     }
 }
 
-// The nine digit sums (exact integers in FP32) as one double, sum_d acc_d 128^-d: two
+// The nine digit sums (integers in FP32) as one double, sum_d acc_d 128^-d: two
 // 64-bit integers below 2^51, each made a double by placing it in the mantissa of a number
 // whose last place has its weight (2^-28, 2^-56), and one add.  Three FP64 adds in all.
 __device__ __forceinline__ double join_digits(const uint32_t (&v)[kSlices][8], int c) {

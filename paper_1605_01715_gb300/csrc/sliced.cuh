@@ -5,9 +5,11 @@
 // exact for entries down to 2^-9 of the largest.  n is written in balanced base-128 digits
 // n = sum_s digit_s 128^(8 - s), digit_s in [-64, 64]: nine FP16 slices of small integers.  A
 // product of two vectors is then a sum over slice pairs (i, j) of integer dot products.  Those
-// with i + j <= 8 are kept, summed by d = i + j: at most 9 pairs x 448 columns x 2^12 < 2^24,
-// so nine FP32 accumulators of the tensor core hold them exactly, whatever it does to bits
-// below its last place.  The accumulators are combined in 64-bit integers and two FP64 terms.
+// with i + j <= 8 are kept, summed by d = i + j: for d <= 7 at most 8 pairs x 512 columns x 2^12 =
+// 2^24, so FP32 accumulators of the tensor core hold them exactly, whatever it does to bits below
+// its last place.  (The last, of 9 pairs, could pass 2^24 and lose a unit or two an MMA, 2^-68 of
+// the largest products each: far below what is left out.)  The accumulators are combined in
+// 64-bit integers and two FP64 terms.
 //
 // Error per column, for |a| < 2^ea and |b| < 2^eb: 2^-62 of 2^(ea + eb) from the fixed point,
 // and at most 1.008 x 2^-60 from the pairs left out (eight with i + j = 9 of 2^12 x 128^7 each,

@@ -195,7 +195,7 @@ def test_product_is_exact_to_its_bound(make, K, M, n):
     rng = np.random.default_rng(K)
     a, b = make(rng, M, n, K)
     got = _product(a[None], b, M, [(0, np.arange(n), np.arange(n))])
-    exact, chunks = _exact(a, b, 448)
+    exact, chunks = _exact(a, b, 512)
     err, bound = np.abs(got - exact), _bound(a, b, exact, chunks)
     print("K=%d M=%d n=%d worst error / bound %.3f" % (K, M, n, float((err / bound).max())))
     assert (err <= bound).all()
