@@ -2900,8 +2900,8 @@ int matvec(Plan& P, const Bufs<Real>& B, const double* q, double* out, cudaStrea
     if (std::is_same<Real, float>::value) {
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
         KF_CHECK_CUDA(cudaStreamIsCapturing(s, &cap));
-        P.pdl = chain_early(cap == cudaStreamCaptureStatusActive, P.kernel, P.near_pairs, P.n_p2l > 0, P.n_p2p_units,
-                            P.near_resident);
+        P.pdl = chain_early(cap == cudaStreamCaptureStatusActive, P.kernel, P.near_pairs, P.n_p2l > 0,
+                            warp_near(P) ? P.n_p2p_units : 0, P.near_resident);
     }
     KF_TRY(mark(0));
     if (near_overlap) {

@@ -70,9 +70,11 @@ struct OpTables {
 // 213).  In a captured graph there are no such gaps, and the waiting blocks of the translation
 // kernel hold whole SMs that a near field of many pairs, or of more than a wave of units (resident:
 // the warps the chip holds) beside an X list, would use.  Of 380 such plans the 286 that take it
-// gain 3 % on average (at most 16), the others below 50M pairs would lose 7 % (at most 25): double
-// layer of 120,000 points 209 / 228 us, of 25,920 at 192 a leaf 183 / 223, single layer of 72,000
-// (33M pairs, 1.7 waves) 208 / 238, 64,000-point pack (41M, 1.5 waves) 303 / 354.
+// gain 3 % on average (at most 16), the others below 50M pairs would lose 7 % (at most 25), most of
+// it to the leaves' projection, which waits for S2U: double layer of 25,920 points at 192 a leaf
+// 183 / 223 us, single layer of 72,000 (33M pairs, 1.7 waves) 208 / 238, 64,000-point pack (41M,
+// 1.5 waves) 303 / 354.  The block kernel has no units, and its plans gain up to 50M pairs (38,720
+// points at 96 a leaf 151 / 142).
 inline bool chain_early(bool captured, int kernel, int64_t near_pairs, bool x_list, int64_t units, int64_t resident) {
     const bool dl = kernel == KIFMM_KERNEL_DL;
     if (!captured) return near_pairs < 50000000;

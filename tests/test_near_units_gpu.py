@@ -50,7 +50,7 @@ def test_pass_width(kernel, p, freq, leaf):
     ("dl", 3.6e6, 0, 628, True, True), ("sl", 11.1e6, 0, 2236, True, True), ("adl", 14.8e6, 1, 1348, True, True),
     ("sl", 30.7e6, 1, 2072, True, True), ("dl", 11.6e6, 0, 3248, True, True), ("sl", 23.5e6, 0, 5816, True, True),
     ("dl", 31.0e6, 0, 4864, True, False), ("sl", 32.6e6, 1, 4232, True, False), ("dl", 37.4e6, 0, 1784, True, False),
-    ("dl", 17.2e6, 1, 4880, True, False), ("adl", 40.9e6, 1, 3546, True, False), ("sl", 77.2e6, 1, 2440, False, False),
+    ("dl", 17.2e6, 1, 4880, True, False), ("sl", 24.7e6, 1, 0, True, True), ("adl", 40.9e6, 1, 3546, True, False), ("sl", 77.2e6, 1, 2440, False, False),
     ("adl", 628.3e6, 1, 33792, False, False),
 ])
 def test_early_launch_rule(kernel, pairs, x_list, units, direct, captured):
